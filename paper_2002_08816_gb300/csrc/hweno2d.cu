@@ -21,8 +21,10 @@
 //      fluxes at the 4 ng interface points, Eq. (ode2) and Eq. (RK);
 //   5. the tile's wave-speed maxima (x and y) into the slots for the next
 //      stage, the troubled count and the status bits.
-// The reconstruction arithmetic is the generated straight-line code of
-// hweno2d_coef.cuh (square cells); the FP32 Euler kernel runs it, the fluxes
+// The reconstruction arithmetic is generated straight-line code (square cells):
+// the linear p0 by parity classes (hweno2d_sym.cuh, which gives what that
+// saves), the HWENO candidates and smoothness indicators of
+// hweno2d_coef.cuh; the FP32 Euler kernel runs it, the fluxes
 // and the HWENO helpers on pairs (two components, two points or two
 // characteristic fields) in packed FP32 (fma.rn.f32x2).
 #include <cuda.h>
@@ -234,6 +236,41 @@ __device__ __forceinline__ void store_point(S& sm, int c, int p, int ci, int cj,
     sm.xf[c][p][cj][ci + 1] = v;        // left and right faces
   else
     sm.yf[c][p - NG2][cj + 1][ci] = v;  // bottom and top faces
+}
+
+template <typename S>
+__device__ __forceinline__ void store_points(S& sm, int c, int p, int ci, int cj, float2 v) {
+  store_point(sm, c, p, ci, cj, v.x);
+  store_point(sm, c + 1, p, ci, cj, v.y);
+}
+template <typename S, typename R>
+__device__ __forceinline__ void store_points(S& sm, int c, int p, int ci, int cj, R v) {
+  store_point(sm, c, p, ci, cj, v);
+}
+
+// What the linear maps take per step: two FP32 components, or one value.
+template <typename R, bool PACKED>
+struct PairOf { typedef R type; };
+template <>
+struct PairOf<float, true> { typedef float2 type; };
+
+// The parity classes (hw2::p0_classes) of component c of the cell at own-tile
+// coordinates (ci, cj), PACKED: of components c and c + 1.
+template <bool COMP, bool PACKED, typename S, typename T>
+__device__ __forceinline__ void classes_of(const S& sm, int c, int ci, int cj, T* s) {
+  if constexpr (PACKED) {
+    float da[19], db[19];
+    gather_data<COMP>(sm, c, ci, cj, da);
+    gather_data<COMP>(sm, c + 1, ci, cj, db);
+    float2 d[19];
+#pragma unroll
+    for (int k = 0; k < 19; ++k) d[k] = make_float2(da[k], db[k]);
+    hw2::p0_classes(d, s);
+  } else {
+    T d[19];
+    gather_data<COMP>(sm, c, ci, cj, d);
+    hw2::p0_classes(d, s);
+  }
 }
 
 // Step 5.1 for an Euler cell whose 3x3 stencil holds a troubled cell: the
@@ -573,11 +610,11 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
     if (item < TX * TY) {  // own cell: every interface point
       ci = item % TX; cj = item / TX; p_lo = 0; p_hi = NF;
     } else {               // cross halo: the one face shared with the tile
-      const int h = item - TX * TY;
-      if (h < TY) { ci = -1; cj = h; p_lo = NG; p_hi = 2 * NG; }
-      else if (h < 2 * TY) { ci = TX; cj = h - TY; p_lo = 0; p_hi = NG; }
-      else if (h < 2 * TY + TX) { ci = h - 2 * TY; cj = -1; p_lo = 3 * NG; p_hi = 4 * NG; }
-      else { ci = h - 2 * TY - TX; cj = TY; p_lo = 2 * NG; p_hi = 3 * NG; }
+      const int h = item - TX * TY;  // the y-faces first: a warp has items of one kind
+      if (h < TX) { ci = h; cj = -1; p_lo = 3 * NG; p_hi = 4 * NG; }
+      else if (h < 2 * TX) { ci = h - TX; cj = TY; p_lo = 2 * NG; p_hi = 3 * NG; }
+      else if (h < 2 * TX + TY) { ci = -1; cj = h - 2 * TX; p_lo = NG; p_hi = 2 * NG; }
+      else { ci = TX; cj = h - 2 * TX - TY; p_lo = 0; p_hi = NG; }
     }
   };
   for (int item = tid; item < TX * TY + 2 * TX + 2 * TY; item += NT) {
@@ -591,33 +628,26 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
         for (int di = -1; di <= 1; ++di) hw |= sm.fl[cj + 2 + dj][ci + 2 + di] != 0;
     }
     if (!hw) {
-      if constexpr (kPacked) {
-        // FP32 Euler: components (0, 1) and (2, 3) through the packed map
+      // the classes of one component, or (FP32 Euler) of components c and
+      // c + 1 at once, then the face pairs the item needs
+      using T = typename PairOf<R, kPacked>::type;
 #pragma unroll
-        for (int c = 0; c < C; c += 2) {
-          R da[19], db[19];
-          gather_data<COMP>(sm, c, ci, cj, da);
-          gather_data<COMP>(sm, c + 1, ci, cj, db);
-          float2 d2[19], v2[NF];
+      for (int c = 0; c < C; c += kPacked ? 2 : 1) {
+        T s[19];
+        classes_of<COMP, kPacked>(sm, c, ci, cj, s);
+        if (p_lo < 2 * NG) {
+          T v[2 * NG];
+          p0s_xfaces<NG>(s, v);
 #pragma unroll
-          for (int k = 0; k < 19; ++k) d2[k] = make_float2(da[k], db[k]);
-          p0_faces_x2<NG>(d2, v2);
-#pragma unroll
-          for (int p = 0; p < NF; ++p)
-            if (p >= p_lo && p < p_hi) {
-              store_point(sm, c, p, ci, cj, v2[p].x);
-              store_point(sm, c + 1, p, ci, cj, v2[p].y);
-            }
+          for (int p = 0; p < 2 * NG; ++p)
+            if (p >= p_lo && p < p_hi) store_points(sm, c, p, ci, cj, v[p]);
         }
-      } else {
+        if (p_hi > 2 * NG) {
+          T v[2 * NG];
+          p0s_yfaces<NG>(s, v);
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-          R d[19], v[NF];
-          gather_data<COMP>(sm, c, ci, cj, d);
-          p0_faces<NG>(d, v);
-#pragma unroll
-          for (int p = 0; p < NF; ++p)
-            if (p >= p_lo && p < p_hi) store_point(sm, c, p, ci, cj, v[p]);
+          for (int p = 0; p < 2 * NG; ++p)
+            if (p + 2 * NG >= p_lo && p + 2 * NG < p_hi) store_points(sm, c, p + 2 * NG, ci, cj, v[p]);
         }
       }
     }
@@ -686,28 +716,22 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
 #pragma unroll
     for (int c = 0; c < C; ++c) Fv[c] = Gv[c] = R(0);
     R inter[C][NI];
-    if constexpr (kPacked) {
+    {
+      using T = typename PairOf<R, kPacked>::type;
 #pragma unroll
-      for (int c = 0; c < C; c += 2) {
-        R da[19], db[19];
-        gather_data<COMP>(sm, c, ci, cj, da);
-        gather_data<COMP>(sm, c + 1, ci, cj, db);
-        float2 d2[19], i2[NI];
-#pragma unroll
-        for (int k = 0; k < 19; ++k) d2[k] = make_float2(da[k], db[k]);
-        p0_interior_x2<NG>(d2, i2);
+      for (int c = 0; c < C; c += kPacked ? 2 : 1) {
+        T s[19], v[NI];
+        classes_of<COMP, kPacked>(sm, c, ci, cj, s);
+        p0s_interior<NG>(s, v);
 #pragma unroll
         for (int l = 0; l < NI; ++l) {
-          inter[c][l] = i2[l].x;
-          inter[c + 1][l] = i2[l].y;
+          if constexpr (kPacked) {
+            inter[c][l] = v[l].x;
+            inter[c + 1][l] = v[l].y;
+          } else {
+            inter[c][l] = v[l];
+          }
         }
-      }
-    } else {
-#pragma unroll
-      for (int c = 0; c < C; ++c) {
-        R d[19];
-        gather_data<COMP>(sm, c, ci, cj, d);
-        p0_interior<NG>(d, inter[c]);
       }
     }
     // the volume integrals of Eq. (ode2) at interior point p (weight

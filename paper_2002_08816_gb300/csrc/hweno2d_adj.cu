@@ -410,11 +410,11 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
       R da[19], db[19];
       gather19a(sm, c, ci, cj, da);
       gather19a(sm, c + 1, ci, cj, db);
-      float2 d2[19], v2[NP];
+      float2 d2[19], s2[19], v2[NP];
 #pragma unroll
       for (int k = 0; k < 19; ++k) d2[k] = make_float2(da[k], db[k]);
-      p0_faces_x2<NG>(d2, v2);
-      p0_interior_x2<NG>(d2, &v2[NF]);
+      hw2::p0_classes(d2, s2);
+      p0s_points<NG>(s2, v2);
 #pragma unroll
       for (int p = 0; p < NP; ++p) {
         P[c][p] = v2[p].x;
@@ -424,10 +424,10 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
   } else {
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-      R d[19];
+      R d[19], s[19];
       gather19a(sm, c, ci, cj, d);
-      p0_faces<NG>(d, P[c]);
-      p0_interior<NG>(d, &P[c][NF]);
+      hw2::p0_classes(d, s);
+      p0s_points<NG>(s, P[c]);
       if constexpr (C == 1) {
         if (hw) hweno2d_faces<NG>(d, P_.gam, P_.eps, 0, NF, P[c]);
       }
@@ -609,13 +609,17 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
         float2 l2[NP];
 #pragma unroll
         for (int p = 0; p < NP; ++p) l2[p] = make_float2(P[c][p], P[c + 1][p]);
+        float2 s2[19];
+#pragma unroll
+        for (int k = 0; k < 19; ++k) s2[k] = make_float2(0.0f, 0.0f);
         if (!hw) {
-          p0_faces_T_x2<NG>(l2, g2);
+          p0s_faces_T<NG>(l2, s2);
         } else {
 #pragma unroll
           for (int k = 0; k < 19; ++k) g2[k] = make_float2(Gl[c][k], Gl[c + 1][k]);
         }
-        p0_interior_T_x2<NG>(&l2[NF], g2);
+        p0s_interior_T<NG>(&l2[NF], s2);
+        hw2::p0_classes_T(s2, g2);
       }
       // both components' tile sums at once (each in the fixed order of the
       // single-component exchange)
@@ -667,8 +671,11 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
 #pragma unroll
       for (int k = 0; k < 19; ++k) g[k] = R(0);
       if (own) {
+        R s[19];
+#pragma unroll
+        for (int k = 0; k < 19; ++k) s[k] = R(0);
         if (!hw) {
-          p0_faces_T<NG>(P[c], g);
+          p0s_faces_T<NG>(P[c], s);
         } else if constexpr (C == 1) {
           R d[19];
           gather19a(sm, c, ci, cj, d);
@@ -677,7 +684,8 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
 #pragma unroll
           for (int k = 0; k < 19; ++k) g[k] = Gl[c][k];
         }
-        p0_interior_T<NG>(&P[c][NF], g);
+        p0s_interior_T<NG>(&P[c][NF], s);
+        hw2::p0_classes_T(s, g);
       }
       exchange(c, g);
     }

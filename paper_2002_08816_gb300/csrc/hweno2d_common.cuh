@@ -7,6 +7,7 @@
 
 #include "hweno1d_recon.cuh"
 #include "hweno2d_coef.cuh"
+#include "hweno2d_sym.cuh"
 
 namespace hw {
 
@@ -208,18 +209,33 @@ template <int NG, typename R>
 __device__ __forceinline__ void p0_faces(const R* d, R* o) {
   if constexpr (NG == 3) hw2::p0_faces_ng3(d, o); else hw2::p0_faces_ng2(d, o);
 }
-template <int NG, typename R>
-__device__ __forceinline__ void p0_interior(const R* d, R* o) {
-  if constexpr (NG == 3) hw2::p0_interior_ng3(d, o); else hw2::p0_interior_ng2(d, o);
-}
-// The same two maps on two components of a cell at once (packed FP32).
+// The same map on two components of a cell at once (packed FP32).
 template <int NG>
 __device__ __forceinline__ void p0_faces_x2(const float2* d, float2* o) {
   if constexpr (NG == 3) hw2::p0_faces_ng3_x2(d, o); else hw2::p0_faces_ng2_x2(d, o);
 }
-template <int NG>
-__device__ __forceinline__ void p0_interior_x2(const float2* d, float2* o) {
-  if constexpr (NG == 3) hw2::p0_interior_ng3_x2(d, o); else hw2::p0_interior_ng2_x2(d, o);
+// The linear p0 of one component (T = float, double) or of two at once (float2)
+// from its parity classes s (hw2::p0_classes of the 19 data): the 2 NG values
+// on the left and right faces, on the bottom and top faces, and the NG^2
+// interior values.
+template <int NG, typename T>
+__device__ __forceinline__ void p0s_xfaces(const T* s, T* o) {
+  if constexpr (NG == 3) hw2::p0s_xfaces_ng3(s, o); else hw2::p0s_xfaces_ng2(s, o);
+}
+template <int NG, typename T>
+__device__ __forceinline__ void p0s_yfaces(const T* s, T* o) {
+  if constexpr (NG == 3) hw2::p0s_yfaces_ng3(s, o); else hw2::p0s_yfaces_ng2(s, o);
+}
+template <int NG, typename T>
+__device__ __forceinline__ void p0s_interior(const T* s, T* o) {
+  if constexpr (NG == 3) hw2::p0s_interior_ng3(s, o); else hw2::p0s_interior_ng2(s, o);
+}
+// every point value, in the order of hweno2d_coef.cuh
+template <int NG, typename T>
+__device__ __forceinline__ void p0s_points(const T* s, T* o) {
+  p0s_xfaces<NG>(s, o);
+  p0s_yfaces<NG>(s, o + 2 * NG);
+  p0s_interior<NG>(s, o + 4 * NG);
 }
 template <int NG, typename R>
 __device__ __forceinline__ void q_faces(int n, const R* d, R* o) {

@@ -117,18 +117,22 @@ template <int NG, typename R>
 __device__ __forceinline__ void p0_faces_T(const R* l, R* g) {
   if constexpr (NG == 3) hw2::p0_faces_ng3_T(l, g); else hw2::p0_faces_ng2_T(l, g);
 }
-template <int NG, typename R>
-__device__ __forceinline__ void p0_interior_T(const R* l, R* g) {
-  if constexpr (NG == 3) hw2::p0_interior_ng3_T(l, g); else hw2::p0_interior_ng2_T(l, g);
+// The transposes of the parity-class maps (T one component, or float2: two):
+// the adjoints of the interface (interior) values added to those of the
+// classes (hw2::p0_classes_T sends them back to the 19 data).
+template <int NG, typename T>
+__device__ __forceinline__ void p0s_faces_T(const T* l, T* s) {
+  if constexpr (NG == 3) {
+    hw2::p0s_xfaces_ng3_T(l, s);
+    hw2::p0s_yfaces_ng3_T(l + 2 * NG, s);
+  } else {
+    hw2::p0s_xfaces_ng2_T(l, s);
+    hw2::p0s_yfaces_ng2_T(l + 2 * NG, s);
+  }
 }
-// The same two transposes on two components at once (packed FP32).
-template <int NG>
-__device__ __forceinline__ void p0_faces_T_x2(const float2* l, float2* g) {
-  if constexpr (NG == 3) hw2::p0_faces_ng3_T_x2(l, g); else hw2::p0_faces_ng2_T_x2(l, g);
-}
-template <int NG>
-__device__ __forceinline__ void p0_interior_T_x2(const float2* l, float2* g) {
-  if constexpr (NG == 3) hw2::p0_interior_ng3_T_x2(l, g); else hw2::p0_interior_ng2_T_x2(l, g);
+template <int NG, typename T>
+__device__ __forceinline__ void p0s_interior_T(const T* l, T* s) {
+  if constexpr (NG == 3) hw2::p0s_interior_ng3_T(l, s); else hw2::p0s_interior_ng2_T(l, s);
 }
 template <int NG, typename R>
 __device__ __forceinline__ void q_faces_T(int n, const R* l, R* g) {
