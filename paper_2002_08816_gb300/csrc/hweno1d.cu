@@ -6,7 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "hweno1d_stage.cuh"
+#include "hweno1d_stage64.cuh"
 
 namespace hw {
 namespace {
@@ -19,16 +19,46 @@ constexpr int T = kTile1D;      // their cells per CTA
 constexpr int NW = NT / 32;
 
 // Every CTA has NTH cell threads and one scalar warp (hweno1d_stage.cuh).
-// The 128-thread tiles are the high-occupancy choice: 8 CTAs per SM in FP32
-// (at most 51 registers), 6 in FP64, which hides the stage's dependent
-// load and arithmetic chains on large states and batches; on small states,
-// which sit at the per-stage latency floor, the 256-thread tiles at the
-// register count the compiler picks are faster.  hweno_autotune chooses.
+// FP32: a tile is NTH - 6 cells, a cell per thread; the 128-thread tiles are
+// the high-occupancy choice (8 CTAs per SM, at most 51 registers), which hides
+// the stage's dependent load and arithmetic chains on large states and
+// batches; on small states, which sit at the per-stage latency floor, the
+// 256-thread tiles at the register count the compiler picks are faster.
+// hweno_autotune chooses.  FP64: the tasks of hweno1d_fp64.cuh on the same
+// tiles, and on tiles of 26 cells with 128 threads (nth = 32, stage_nth) for
+// grids that leave SMs idle otherwise.
+template <typename R, int NTH>
+constexpr int tile_cells() { return NTH == 32 ? 26 : NTH - 2 * H; }
+template <typename R, int NTH>
+constexpr int cell_threads() { return NTH == 32 ? 128 : NTH; }
+template <typename R, int NTH>
+constexpr int min_ctas() {
+  return sizeof(R) == 4 ? (NTH == 128 ? 8 : 1) : (NTH <= 128 ? 4 : NTH == 256 ? 2 : 1);
+}
+
+// One tile of one stage; the tile's arrays are in dynamic shared memory.
 template <typename R, int C, bool BATCH, int NTH>
-__global__ void __launch_bounds__(NTH + 32, NTH == 128 ? (sizeof(R) == 4 ? 8 : 6) : 1)
+struct StageTile {
+  typedef Smem1D<R, C, NTH> Smem;
+  static __device__ __forceinline__ void run(const Stage1DArgs& a, int tile, Smem& sm) {
+    s1d::stage1d_tile<R, C, BATCH, NTH>(a, tile, sm);
+  }
+};
+template <int C, bool BATCH, int NTH>
+struct StageTile<double, C, BATCH, NTH> {
+  static constexpr int T = tile_cells<double, NTH>(), N = cell_threads<double, NTH>();
+  typedef f64::Smem64<C, T> Smem;
+  static __device__ __forceinline__ void run(const Stage1DArgs& a, int tile, Smem& sm) {
+    f64::stage64_tile<C, BATCH, T, N>(a, tile, sm);
+  }
+};
+
+template <typename R, int C, bool BATCH, int NTH>
+__global__ void __launch_bounds__(cell_threads<R, NTH>() + 32, min_ctas<R, NTH>())
     stage1d_kernel(Stage1DArgs a) {
-  __shared__ Smem1D<R, C, NTH> sm;
-  s1d::stage1d_tile<R, C, BATCH, NTH>(a, blockIdx.x, sm);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  typedef StageTile<R, C, BATCH, NTH> Tile;
+  Tile::run(a, blockIdx.x, *reinterpret_cast<typename Tile::Smem*>(smem_raw));
 }
 
 // ------------------------------------------------------------ persistent run
@@ -95,7 +125,9 @@ __global__ void __launch_bounds__(128) barrier_check_kernel(unsigned* bar, int m
 
 template <typename R, int C, bool BATCH, int NTH>
 __global__ void __launch_bounds__(NTH + 32) run1d_kernel(Run1DArgs r) {
-  __shared__ Smem1D<R, C, NTH> sm;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  typedef StageTile<R, C, BATCH, NTH> Tile;
+  typename Tile::Smem& sm = *reinterpret_cast<typename Tile::Smem*>(smem_raw);
   unsigned meet = 0;  // arrivals that end the next meeting
   for (int step = 0; step < r.nsteps; ++step) {
 #pragma unroll 1
@@ -111,7 +143,7 @@ __global__ void __launch_bounds__(NTH + 32) run1d_kernel(Run1DArgs r) {
       a.u0 = stage == 1 ? nullptr : r.W0;
       a.lim_out = stage == 1 ? r.W0 : nullptr;
       for (int tile = blockIdx.x; tile < a.ntile; tile += gridDim.x) {
-        s1d::stage1d_tile<R, C, BATCH, NTH>(a, tile, sm);
+        Tile::run(a, tile, sm);
         __syncthreads();
       }
       meet += gridDim.x;
@@ -120,12 +152,21 @@ __global__ void __launch_bounds__(NTH + 32) run1d_kernel(Run1DArgs r) {
   }
 }
 
+// Dynamic shared memory beyond 48 KB has to be allowed per kernel.
+template <typename K>
+cudaError_t allow_smem(K kernel, size_t bytes) {
+  if (bytes <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 template <typename R, int C, bool BATCH, int NTH>
 cudaError_t max_ctas_t(int* ctas) {
+  constexpr size_t smem = sizeof(typename StageTile<R, C, BATCH, NTH>::Smem);
   int dev = 0, nsm = 0, per = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, run1d_kernel<R, C, BATCH, NTH>, NTH + 32, 0);
+  if (e == cudaSuccess) e = allow_smem(run1d_kernel<R, C, BATCH, NTH>, smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, run1d_kernel<R, C, BATCH, NTH>, NTH + 32, smem);
   *ctas = per * nsm;
   return e;
 }
@@ -142,7 +183,8 @@ cudaError_t run_t(const Run1DArgs& r, cudaStream_t s) {
   Run1DArgs rc = r;
   void* args[] = {&rc};
   return cudaLaunchCooperativeKernel((const void*)run1d_kernel<R, C, BATCH, NTH>, dim3(grid),
-                                     dim3(NTH + 32), args, 0, s);
+                                     dim3(NTH + 32), args,
+                                     sizeof(typename StageTile<R, C, BATCH, NTH>::Smem), s);
 }
 
 template <typename R, int C, bool BATCH>
@@ -156,19 +198,6 @@ template <typename R, int C>
 cudaError_t run_c(const Run1DArgs& r, cudaStream_t s) {
   return r.a.tile_inst ? run_b<R, C, true>(r, s) : run_b<R, C, false>(r, s);
 }
-
-template <typename R, int C, bool BATCH>
-cudaError_t max_b(int nth, int* ctas) {
-  if (nth == 128) return max_ctas_t<R, C, BATCH, 128>(ctas);
-  if (nth == 512) return max_ctas_t<R, C, BATCH, 512>(ctas);
-  return max_ctas_t<R, C, BATCH, 256>(ctas);
-}
-
-template <typename R, int C>
-cudaError_t max_c(int batch, int nth, int* ctas) {
-  return batch ? max_b<R, C, true>(nth, ctas) : max_b<R, C, false>(nth, ctas);
-}
-
 
 // Wave-speed maxima in FP64 slots (the per-cell speeds in the kernel's
 // precision, as the stage kernels compute them).
@@ -302,27 +331,37 @@ __global__ void set_scalars_kernel(DevScalars* sc, int reset, double t_final) {
 
 // Stage launches allow programmatic dependent launch: a stage's CTAs can be
 // resident before the previous stage ends and start at its completion.
-template <typename R, int C, int NTH>
+template <typename R, int C, bool BATCH, int NTH>
 cudaError_t launch_stage1d_n(const Stage1DArgs& a, cudaStream_t s) {
+  constexpr size_t smem = sizeof(typename StageTile<R, C, BATCH, NTH>::Smem);
+  cudaError_t e = allow_smem(stage1d_kernel<R, C, BATCH, NTH>, smem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)a.ntile);
-  cfg.blockDim = dim3(NTH + 32);
-  cfg.dynamicSmemBytes = 0;
+  cfg.blockDim = dim3(cell_threads<R, NTH>() + 32);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (a.tile_inst) return cudaLaunchKernelEx(&cfg, stage1d_kernel<R, C, true, NTH>, a);
-  return cudaLaunchKernelEx(&cfg, stage1d_kernel<R, C, false, NTH>, a);
+  return cudaLaunchKernelEx(&cfg, stage1d_kernel<R, C, BATCH, NTH>, a);
+}
+
+template <typename R, int C, bool BATCH>
+cudaError_t launch_stage1d_b(const Stage1DArgs& a, cudaStream_t s) {
+  if constexpr (sizeof(R) == 8 && !BATCH) {
+    if (a.nth == 32) return launch_stage1d_n<R, C, BATCH, 32>(a, s);
+  }
+  if (a.nth == 128) return launch_stage1d_n<R, C, BATCH, 128>(a, s);
+  if (a.nth == 512) return launch_stage1d_n<R, C, BATCH, 512>(a, s);
+  return launch_stage1d_n<R, C, BATCH, 256>(a, s);
 }
 
 template <typename R, int C>
 cudaError_t launch_stage1d_t(const Stage1DArgs& a, cudaStream_t s) {
-  if (a.nth == 128) return launch_stage1d_n<R, C, 128>(a, s);
-  if (a.nth == 512) return launch_stage1d_n<R, C, 512>(a, s);
-  return launch_stage1d_n<R, C, 256>(a, s);
+  return a.tile_inst ? launch_stage1d_b<R, C, true>(a, s) : launch_stage1d_b<R, C, false>(a, s);
 }
 
 template <typename R, int C>
@@ -333,11 +372,6 @@ void alpha1d_batch_t(const Stage1DArgs& a, cudaStream_t s) {
 }
 
 }  // namespace
-
-cudaError_t run1d_max_ctas(int system, int fp64, int batch, int nth, int* ctas) {
-  if (system == 0) return fp64 ? max_c<double, 1>(batch, nth, ctas) : max_c<float, 1>(batch, nth, ctas);
-  return fp64 ? max_c<double, 3>(batch, nth, ctas) : max_c<float, 3>(batch, nth, ctas);
-}
 
 cudaError_t launch_run1d(const Run1DArgs& r, cudaStream_t s) {
   if (r.a.system == 0) return r.a.fp64 ? run_c<double, 1>(r, s) : run_c<float, 1>(r, s);

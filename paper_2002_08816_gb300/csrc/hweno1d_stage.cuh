@@ -335,33 +335,32 @@ __device__ __forceinline__ void rhs_parts_of_cell(const Smem1D<R, C, NTH>& sm, i
   }
 }
 
-// One stage on one tile of T = NTH - 6 cells, by a CTA of NTH + 32 threads.  The
-// per-stage kernel calls it once; the persistent kernel calls it for each of
-// its tiles of each stage, between grid barriers, so every load of data
-// produced in the same launch goes through L2 (ldx).
-template <typename R, int C, bool BATCH, int NTH>
-__device__ __forceinline__ void stage1d_tile(Stage1DArgs a, const int tile, Smem1D<R, C, NTH>& sm) {
-  constexpr int T = NTH - 2 * H, NT = NTH, NW = NTH / 32;
-  const int tid = threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
-  int n = a.n;
-  int base = tile * T;
-  int inst = 0;
-  bool lead = tile == 0;  // the tile that keeps the (instance's) time
+// Where a tile lies: its cells base .. of the instance's n, and whether it keeps
+// the (instance's) time.
+struct TileAt {
+  int n, base, inst;
+  bool lead;
+};
+
+// The tile's place (tiles of T cells), and for a batch the arguments moved to
+// its instance.
+template <typename R, int C, bool BATCH>
+__device__ __forceinline__ TileAt tile_at(Stage1DArgs& a, int tile, int T) {
+  TileAt x = {a.n, tile * T, 0, tile == 0};
   if constexpr (BATCH) {
     // a batch of independent instances: this tile's instance and first cell
-    inst = a.tile_inst[tile];
-    base = a.tile_base[tile];
-    const BatchInst& bi = a.binst[inst];
-    n = bi.n;
-    lead = base == 0;
+    x.inst = a.tile_inst[tile];
+    x.base = a.tile_base[tile];
+    const BatchInst& bi = a.binst[x.inst];
+    x.n = bi.n;
+    x.lead = x.base == 0;
     const long long off = bi.off;
     a.w = static_cast<const R*>(a.w) + off;
     if (a.u0) a.u0 = static_cast<const R*>(a.u0) + off;
     a.out = static_cast<R*>(a.out) + off;
     if (a.lim_out) a.lim_out = static_cast<R*>(a.lim_out) + off;
     if (a.flags_out) a.flags_out += off / (2 * C);
-    a.a_in = static_cast<const double*>(a.a_in) + inst;
+    a.a_in = static_cast<const double*>(a.a_in) + x.inst;
     a.nin = 1;
     a.inv_dx = bi.inv_dx;
     a.h = bi.h;
@@ -371,6 +370,121 @@ __device__ __forceinline__ void stage1d_tile(Stage1DArgs a, const int tile, Smem
     a.f32[5] = bi.inv_dx_f;
     a.f32[6] = bi.cfl_dx_f;
   }
+  return x;
+}
+
+// The scalar warp of a tile: alpha, dt and the time, in FP64; alpha and dt go to
+// the cell threads through shared memory and kBarAll (it only arrives there).
+template <typename R, bool BATCH>
+__device__ __forceinline__ void scalar_warp(const Stage1DArgs& a, int tile, int inst, bool lead, int lane,
+                                            int nt, R* alpha_out, R* dt_out) {
+  // its own loads go out first, concurrently with the cell threads' tile
+  const unsigned long long* a_in = static_cast<const unsigned long long*>(a.a_in);
+  unsigned long long am = 0ull;  // bit patterns of non-negative doubles: the
+                                 // integer order is the numeric order
+  for (int k = lane; k < a.nin; k += 32) {
+    const unsigned long long v = ldx(a_in + k);
+    am = v > am ? v : am;
+  }
+  double rem = 0.0, dt = 0.0, tf = 0.0, t = 0.0;
+  unsigned last = 0u;
+  unsigned long long steps = 0ull;
+  const bool keep = a.stage == 3 && lead && lane == 0;  // the time keeper
+  if constexpr (BATCH) {
+    const BatchScalars& bs = a.bsc[inst];
+    if (a.stage == 1) rem = ldx(&bs.rem);
+    else if (a.stage > 1) dt = ldx(&bs.dt);
+    if (keep) {
+      last = ldx(&bs.last);
+      t = ldx(&bs.t);
+    }
+  } else {
+    if (a.stage == 1) rem = ldx(&a.sc->rem);
+    else if (a.stage > 1) dt = ldx(&a.sc->dt);
+    if (keep) {
+      last = ldx(&a.sc->last);
+      t = ldx(&a.sc->t);
+    }
+  }
+  if (keep) {
+    tf = ldx(&a.sc->t_final);
+    steps = ldx(&a.sc->steps);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long v = __shfl_xor_sync(0xffffffffu, am, o);
+    am = v > am ? v : am;
+  }
+  asm volatile("griddepcontrol.launch_dependents;");
+  const double alpha = __longlong_as_double((long long)am);
+  if (a.stage == 1) {
+    // dt = CFL dx / alpha(u^n), clipped to the remaining time (the clipped
+    // step is the last one and ends exactly at t_final); 0 once t_final
+    // has been reached
+    dt = a.cfl_dx / alpha;
+    last = 0u;
+    if (rem <= 0.0) {
+      dt = 0.0;
+    } else if (dt >= rem) {
+      dt = rem;
+      last = 1u;
+    }
+    if (!(alpha > 0.0) || !isfinite(dt)) dt = 0.0;
+    if (lead && lane == 0) {
+      if constexpr (BATCH) {
+        BatchScalars& bs = a.bsc[inst];
+        bs.dt = dt;
+        bs.dt_f = (float)dt;
+        bs.last = last;
+      } else {
+        a.sc->dt = dt;
+        a.sc->dt_f = (float)dt;
+        a.sc->last = last;
+      }
+    }
+  }
+  if (lane == 0) {
+    *alpha_out = R(alpha);
+    *dt_out = R(dt);
+  }
+  if (a.stage > 0 && dt > 0.0) {
+    // the slots of the stage after next (read two stages ago, now free)
+    if constexpr (BATCH) {
+      if (a.a_zero && lead && lane == 0) static_cast<double*>(a.a_zero)[inst] = 0.0;
+    } else {
+      if (a.a_zero && tile == 0)
+        for (int k = lane; k < kAlphaSlots; k += 32) static_cast<double*>(a.a_zero)[k] = 0.0;
+    }
+    if (keep) {  // stage 3 of the lead tile: the step is complete
+      const double tn = last ? tf : t + dt;
+      const double r = tf > 0.0 ? tf - tn : (double)INFINITY;
+      if constexpr (BATCH) {
+        BatchScalars& bs = a.bsc[inst];
+        bs.t = tn;
+        bs.rem = r;
+        bs.rem_f = (float)r;
+        if (inst == 0) a.sc->steps = steps + 1ull;
+      } else {
+        a.sc->t = tn;
+        a.sc->rem = r;
+        a.sc->rem_f = (float)r;
+        a.sc->steps = steps + 1ull;
+      }
+    }
+  }
+  bar_arrive(kBarAll, nt + 32);
+}
+
+// One stage on one tile of T = NTH - 6 cells, by a CTA of NTH + 32 threads.  The
+// per-stage kernel calls it once; the persistent kernel calls it for each of
+// its tiles of each stage, between grid barriers, so every load of data
+// produced in the same launch goes through L2 (ldx).
+template <typename R, int C, bool BATCH, int NTH>
+__device__ __forceinline__ void stage1d_tile(Stage1DArgs a, const int tile, Smem1D<R, C, NTH>& sm) {
+  constexpr int T = NTH - 2 * H, NT = NTH, NW = NTH / 32;
+  const int tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
+  const TileAt at = tile_at<R, C, BATCH>(a, tile, T);
+  const int n = at.n, base = at.base, inst = at.inst;
   const R* __restrict__ w = static_cast<const R*>(a.w);
 
   // The producer of the stage input may still be finishing (programmatic
@@ -388,101 +502,7 @@ __device__ __forceinline__ void stage1d_tile(Stage1DArgs a, const int tile, Smem
   }
 
   if (tid >= NT) {
-    // ---- the scalar warp: alpha, dt and the time, in FP64 ----------------
-    // its own loads go out first, concurrently with the cell threads' tile
-    const unsigned long long* a_in = static_cast<const unsigned long long*>(a.a_in);
-    unsigned long long am = 0ull;  // bit patterns of non-negative doubles: the
-                                   // integer order is the numeric order
-    for (int k = lane; k < a.nin; k += 32) {
-      const unsigned long long v = ldx(a_in + k);
-      am = v > am ? v : am;
-    }
-    double rem = 0.0, dt = 0.0, tf = 0.0, t = 0.0;
-    unsigned last = 0u;
-    unsigned long long steps = 0ull;
-    const bool keep = a.stage == 3 && lead && lane == 0;  // the time keeper
-    if constexpr (BATCH) {
-      const BatchScalars& bs = a.bsc[inst];
-      if (a.stage == 1) rem = ldx(&bs.rem);
-      else if (a.stage > 1) dt = ldx(&bs.dt);
-      if (keep) {
-        last = ldx(&bs.last);
-        t = ldx(&bs.t);
-      }
-    } else {
-      if (a.stage == 1) rem = ldx(&a.sc->rem);
-      else if (a.stage > 1) dt = ldx(&a.sc->dt);
-      if (keep) {
-        last = ldx(&a.sc->last);
-        t = ldx(&a.sc->t);
-      }
-    }
-    if (keep) {
-      tf = ldx(&a.sc->t_final);
-      steps = ldx(&a.sc->steps);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long v = __shfl_xor_sync(0xffffffffu, am, o);
-      am = v > am ? v : am;
-    }
-    asm volatile("griddepcontrol.launch_dependents;");
-    const double alpha = __longlong_as_double((long long)am);
-    if (a.stage == 1) {
-      // dt = CFL dx / alpha(u^n), clipped to the remaining time (the clipped
-      // step is the last one and ends exactly at t_final); 0 once t_final
-      // has been reached
-      dt = a.cfl_dx / alpha;
-      last = 0u;
-      if (rem <= 0.0) {
-        dt = 0.0;
-      } else if (dt >= rem) {
-        dt = rem;
-        last = 1u;
-      }
-      if (!(alpha > 0.0) || !isfinite(dt)) dt = 0.0;
-      if (lead && lane == 0) {
-        if constexpr (BATCH) {
-          BatchScalars& bs = a.bsc[inst];
-          bs.dt = dt;
-          bs.dt_f = (float)dt;
-          bs.last = last;
-        } else {
-          a.sc->dt = dt;
-          a.sc->dt_f = (float)dt;
-          a.sc->last = last;
-        }
-      }
-    }
-    if (lane == 0) {
-      sm.alpha = R(alpha);
-      sm.dt = R(dt);
-    }
-    if (a.stage > 0 && dt > 0.0) {
-      // the slots of the stage after next (read two stages ago, now free)
-      if constexpr (BATCH) {
-        if (a.a_zero && lead && lane == 0) static_cast<double*>(a.a_zero)[inst] = 0.0;
-      } else {
-        if (a.a_zero && tile == 0)
-          for (int k = lane; k < kAlphaSlots; k += 32) static_cast<double*>(a.a_zero)[k] = 0.0;
-      }
-      if (keep) {  // stage 3 of the lead tile: the step is complete
-        const double tn = last ? tf : t + dt;
-        const double r = tf > 0.0 ? tf - tn : (double)INFINITY;
-        if constexpr (BATCH) {
-          BatchScalars& bs = a.bsc[inst];
-          bs.t = tn;
-          bs.rem = r;
-          bs.rem_f = (float)r;
-          if (inst == 0) a.sc->steps = steps + 1ull;
-        } else {
-          a.sc->t = tn;
-          a.sc->rem = r;
-          a.sc->rem_f = (float)r;
-          a.sc->steps = steps + 1ull;
-        }
-      }
-    }
-    bar_arrive(kBarAll, NT + 32);
+    scalar_warp<R, BATCH>(a, tile, inst, at.lead, lane, NT, &sm.alpha, &sm.dt);
     return;
   }
 

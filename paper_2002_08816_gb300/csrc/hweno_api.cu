@@ -37,6 +37,11 @@ struct hweno_ctx {
   int res_tile = 0, res_ncta = 0, res_cap = 0;
   unsigned long long* res_halo = nullptr;     // tagged exchange words of the halos
   unsigned long long* res_entries = nullptr;  // and of the per-CTA maxima
+  // FP64 single instances: the resident run's geometry (tile64 = 0: not
+  // available) and its cross-CTA buffers (allocated on first use)
+  int tile64 = 0, ncta64 = 0;
+  unsigned long long* halo64 = nullptr;
+  unsigned long long* entries64 = nullptr;
   // HWENO_FP32C: the low parts of the averages ([C][n] floats beside U[0]);
   // 1D steps run as the resident launch, 2D steps carry the low parts of the
   // stage buffers U[1], U[2] too (Ulo_s)
@@ -336,6 +341,32 @@ cudaError_t enqueue_resident1d(hweno_ctx* h, int nsteps, cudaStream_t s, int sil
   return hw::launch_resident1d(r, h->nth1d, h->res_ncta, s);
 }
 
+// nsteps Runge-Kutta steps of an FP64 handle in one resident launch.
+cudaError_t enqueue_resident64(hweno_ctx* h, int nsteps, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  if (!h->halo64)
+    e = cudaMalloc(&h->halo64, sizeof(unsigned long long) * hw::resident64_halo_words(h->cfg.system, h->ncta64));
+  if (e == cudaSuccess && !h->entries64)
+    e = cudaMalloc(&h->entries64, sizeof(unsigned long long) * hw::resident64_entry_words(h->ncta64));
+  if (e != cudaSuccess) return e;
+  hw::Resident1DArgs r;
+  memset(&r, 0, sizeof(r));
+  r.a = base_args(h);
+  r.a.sc = h->sc;
+  r.a.w = h->U[0];
+  r.a.out = h->U[0];
+  r.tile = h->tile64;
+  r.nsteps = nsteps;
+  r.part0 = h->part[0];
+  r.part1 = h->part[1];
+  r.halo = h->halo64;
+  r.entries = h->entries64;
+  r.alpha_word = h->entries64 + hw::resident64_entry_words(h->ncta64) - 4;
+  r.polls = 1u << 21;
+  r.silent_cta = -1;
+  return hw::launch_resident64(r, h->ncta64, s);
+}
+
 cudaError_t enqueue_step(hweno_ctx* h, cudaStream_t s) {
   if (h->dim == 2) return enqueue_step2d(h, s);
   hw::Stage1DArgs a = base_args(h);
@@ -628,6 +659,12 @@ hweno_status hweno_create(const hweno_config* cfg, void* cuda_stream, hweno_hand
     hweno_destroy(h);
     return fail(nullptr, HWENO_ERR_CUDA, msg);
   }
+  if (h->dim == 1 && h->esize == 8) e = hw::resident64_geometry(h->n, &h->tile64, &h->ncta64);
+  if (e != cudaSuccess) {
+    std::string msg = std::string("resident launch: ") + cudaGetErrorString(e);
+    hweno_destroy(h);
+    return fail(nullptr, HWENO_ERR_CUDA, msg);
+  }
   if (h->comp && h->dim == 1) {  // the resident launch only
     h->persist1d = 2;
     e = prepare_resident(h);
@@ -698,6 +735,20 @@ hweno_status hweno_step(hweno_handle h, int nsteps, double t_final, double* t_ou
   if (h->n_batch > 0)
     HW_CUDA(h, hw::launch_batch_scalars(h->d_bsc, h->n_batch, 0, t_final, h->stream));
   int left = nsteps;
+  if (h->tile64 > 0 && h->n_batch == 0 && left > 0) {
+    // FP64 single instances whose tiles fit on the GPU at once run on chip,
+    // whatever launch the handle is set to: at every size the FP64 pipe and not
+    // the launches bounds them, and the resident run spreads it best
+    cudaError_t e = enqueue_resident64(h, left, h->stream);
+    if (e == cudaSuccess) {
+      left = 0;
+    } else if (e == cudaErrorCooperativeLaunchTooLarge) {
+      cudaGetLastError();  // fewer SMs than the device has: the other launches
+      h->tile64 = 0;
+    } else {
+      HW_CUDA(h, e);
+    }
+  }
   if (h->dim == 1 && h->persist1d == 2) {
     if (left > 0) HW_CUDA(h, enqueue_resident1d(h, left, h->stream));
     left = 0;
@@ -765,6 +816,7 @@ hweno_status hweno_rhs(hweno_handle h, const void* in, void* out, uint8_t* flags
   a.a_out = nullptr;
   a.sc = h->sc_rhs;
   a.flags_out = flags_out;
+  hw::rhs_tiles1d(a);
   HW_CUDA(h, hw::launch_stage1d(a, h->stream));
   hw::DevScalars s;
   return check_scalars(h, h->sc_rhs, &s);
@@ -834,6 +886,8 @@ void hweno_destroy(hweno_handle h) {
   if (h->bar) cudaFree(h->bar);
   if (h->res_halo) cudaFree(h->res_halo);
   if (h->res_entries) cudaFree(h->res_entries);
+  if (h->halo64) cudaFree(h->halo64);
+  if (h->entries64) cudaFree(h->entries64);
   if (h->Ulo) cudaFree(h->Ulo);
   for (int k = 0; k < 2; ++k)
     if (h->Ulo_s[k]) cudaFree(h->Ulo_s[k]);

@@ -45,7 +45,7 @@ struct Stage1DArgs {
   int n;                 // cells
   int ntile;             // tiles (= CTAs of a per-stage launch)
   int nth;               // threads per CTA of the stage kernels: 128, 256 (also 0) or 512;
-                         // a tile is nth - 6 cells
+                         // a tile is nth - 6 cells (FP64, no batch: also 32, a 26-cell tile)
   int stage;             // 1, 2, 3; 0 = rhs mode
   int bc;                // 0 periodic, 1 outflow
   int mode;              // 0 hybrid, 1 all, 2 none
@@ -185,6 +185,18 @@ cudaError_t prepare_adj2d(int system, int fp64, int ng);
 cudaError_t launch_adj2d(const Adj2DArgs& a, cudaStream_t s);
 
 cudaError_t launch_stage1d(const Stage1DArgs& a, cudaStream_t s);
+// Tiles of one right-hand side evaluation on n cells: a.nth and a.ntile.  FP64
+// on a small grid takes 26-cell tiles (nth = 32): an SM's FP64 pipe is the
+// bound, so the work goes to as many SMs as there are (200 cells, Lax data: the
+// call 79 us on one 250-cell tile with a cell per thread, 42 us on 26-cell
+// ones); from 304 such
+// tiles (two per SM) on, the larger tiles fill the SMs as well.
+inline void rhs_tiles1d(Stage1DArgs& a) {
+  if (a.fp64 && a.n <= 26 * 304) {
+    a.nth = 32;
+    a.ntile = (a.n + 25) / 26;
+  }
+}
 
 // hweno_create's configuration checks (HWENO_OK or HWENO_ERR_ARG; the reason
 // goes to hweno_last_error(NULL)).
@@ -241,8 +253,15 @@ cudaError_t launch_join_pairs(const void* hi, const float* lo, double* out, int 
 // Zeroes the exchange words, then launches.
 cudaError_t launch_resident1d(const Resident1DArgs& r, int nth, int ncta, cudaStream_t s);
 
-// Largest co-resident grid of the persistent kernel for this configuration.
-cudaError_t run1d_max_ctas(int system, int fp64, int batch, int nth, int* ctas);
+// The resident run in FP64 (hweno1d_resident64.cu; single instance, up to
+// two CTAs per SM): its tile and CTAs for n cells (*tile = 0 when the grid does not fit on
+// the GPU at once), the words of its buffers, and the launch, which zeroes
+// them first.  The alpha words (two per parity) follow the entries.
+cudaError_t resident64_geometry(int n, int* tile, int* ncta);
+size_t resident64_entry_words(int ncta);
+size_t resident64_halo_words(int system, int ncta);
+cudaError_t launch_resident64(const Resident1DArgs& r, int ncta, cudaStream_t s);
+
 // Cooperative launch of min(ntile, co-resident CTAs) CTAs.
 cudaError_t launch_run1d(const Run1DArgs& r, cudaStream_t s);
 // hweno_check_barrier's launch; *too_many when ctas cannot all be resident

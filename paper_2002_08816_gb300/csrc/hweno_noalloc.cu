@@ -113,6 +113,7 @@ hweno_status hweno_rhs1d_noalloc(const hweno_config* cfg, void* cuda_stream, con
     a.gas = cfg->gas_gamma;
     for (int k = 0; k < 3; ++k) a.gam[k] = cfg->lin_w[k];
     hw::finish_stage_args(a);
+    hw::rhs_tiles1d(a);
     e = hw::launch_stage1d(a, s);
   }
   unsigned status = 0;
