@@ -467,10 +467,9 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 ? 2 : 1) resident1d_kerne
           ou = su;
           ov = sv;
         } else {
-          const R ca = stage == 2 ? R(0.75) : R(1.0 / 3.0);
           const R cb = stage == 2 ? R(0.25) : R(2.0 / 3.0);
-          ou = ca * u0c[c][0] + cb * su;
-          ov = ca * u0c[c][1] + cb * sv;
+          ou = rk_combine(cb, u0c[c][0], su);
+          ov = rk_combine(cb, u0c[c][1], sv);
         }
         if constexpr (COMP) {
           // the averages: the pair formed before alpha plus the stage's increment

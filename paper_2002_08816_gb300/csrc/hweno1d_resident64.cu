@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(NTH + 32, 2) resident64_kernel(Resident1DArgs 
     f64::lax_friedrichs<C, TMAX, NTH>(sm, Tq, tid, alpha);
     // Eq. (odeH) and Eq. (RK): (component, cell)
     const double kd = dt * par.inv_dx;
-    const double ca = stage == 2 ? 0.75 : 1.0 / 3.0, cb = stage == 2 ? 0.25 : 2.0 / 3.0;
+    const double cb = stage == 2 ? 0.25 : 2.0 / 3.0;
     for (int t = tid; t < C * Tq; t += NTH) {
       const int c = t / Tq, i = t - c * Tq, e = i + H;
       double Gu, Gv;
@@ -285,8 +285,8 @@ __global__ void __launch_bounds__(NTH + 32, 2) resident64_kernel(Resident1DArgs 
         S.u0[c][0][i] = wu;
         S.u0[c][1][i] = wv;
       } else {
-        ou = fma(cb, ou, ca * S.u0[c][0][i]);
-        ov = fma(cb, ov, ca * S.u0[c][1][i]);
+        ou = rk_combine(cb, S.u0[c][0][i], ou);
+        ov = rk_combine(cb, S.u0[c][1][i], ov);
       }
       un[c][0][e] = ou;
       un[c][1][e] = ov;

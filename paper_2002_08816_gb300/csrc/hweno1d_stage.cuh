@@ -624,10 +624,9 @@ __device__ __forceinline__ void stage1d_tile(Stage1DArgs a, const int tile, Smem
           ou = su;
           ov = sv;
         } else {
-          const R ca = a.stage == 2 ? R(0.75) : R(1.0 / 3.0);
           const R cb = a.stage == 2 ? R(0.25) : R(2.0 / 3.0);
-          ou = ca * u0c[c][0] + cb * su;
-          ov = ca * u0c[c][1] + cb * sv;
+          ou = rk_combine(cb, u0c[c][0], su);
+          ov = rk_combine(cb, u0c[c][1], sv);
         }
       }
       R* out = static_cast<R*>(a.out);

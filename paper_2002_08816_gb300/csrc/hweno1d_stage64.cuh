@@ -51,7 +51,7 @@ __device__ __forceinline__ void stage64_tile(Stage1DArgs a, const int tile, Smem
   if (a.stage > 0 && !(dt > 0.0)) return;  // t_final reached: the stage writes nothing
   lax_friedrichs<C, TMAX, NTH>(sm, Tq, tid, alpha);
   const double kd = dt * par.inv_dx;
-  const double ca = a.stage == 2 ? 0.75 : 1.0 / 3.0, cb = a.stage == 2 ? 0.25 : 2.0 / 3.0;
+  const double cb = a.stage == 2 ? 0.25 : 2.0 / 3.0;
   const double* u0 = static_cast<const double*>(a.u0);
   double* out = static_cast<double*>(a.out);
   double* lim = static_cast<double*>(a.lim_out);
@@ -76,8 +76,8 @@ __device__ __forceinline__ void stage64_tile(Stage1DArgs a, const int tile, Smem
       ou = fma(kd, Gu, wu);
       ov = fma(kd, Gv, wv);
       if (a.stage >= 2) {
-        ou = fma(cb, ou, ca * z0);
-        ov = fma(cb, ov, ca * z1);
+        ou = rk_combine(cb, z0, ou);
+        ov = rk_combine(cb, z1, ov);
       }
     }
     out[gu] = ou;

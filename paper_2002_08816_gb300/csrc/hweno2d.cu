@@ -930,9 +930,8 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
           const R s = W[m] + dt * Lm[m];
           if (a.stage == 1) o[m] = s;
           else {
-            const R ca = a.stage == 2 ? R(0.75) : R(1.0 / 3.0);
             const R cb = a.stage == 2 ? R(0.25) : R(2.0 / 3.0);
-            o[m] = ca * u0c[c][m] + cb * s;
+            o[m] = rk_combine(cb, u0c[c][m], s);
           }
         }
         if (!isfinite(o[m])) bad |= ST_NONFINITE;

@@ -70,6 +70,14 @@ __device__ __forceinline__ void atomic_max_nonneg(double* slot, double x) {
             (unsigned long long)__double_as_longlong(x));
 }
 
+// a z + b s of Eq. (RK) with a + b = 1, as z + b (s - z): the rounded 1/3 and 2/3
+// do not add up to one, so that a z + b s moves every average by the same
+// fraction each step (FP32 3e-8, FP64 -6e-17: most of the error of a smooth run).
+template <typename R>
+__device__ __forceinline__ R rk_combine(R b, R z, R s) {
+  return fma(b, s - z, z);
+}
+
 // Ghost cells: periodic wraps, outflow copies the boundary cell.  Any g
 // (a tile's halo may span several periods when n is smaller than a tile).
 __device__ __forceinline__ int bc_map(int g, int n, int bc) {
