@@ -36,6 +36,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "hweno1d_comp.cuh"
 #include "hweno1d_words.cuh"
 
@@ -100,23 +102,52 @@ __device__ __forceinline__ bool poll_word(const u64* p, unsigned tag, u64* out, 
   return false;
 }
 
-template <typename R, int C, int NTH, bool COMP>
+// CL: the CTAs are one thread-block cluster (or a single CTA) and exchange
+// through distributed shared memory instead of words in L2.
+constexpr int kMaxCluster = 16;
+
+template <typename R, int C, int NTH, bool COMP, bool CL>
 struct SmemRes {
+  static constexpr int NV = COMP ? 3 : 2;  // values per cell and component: average, first
+                                           // moment (, low part of the average)
   Smem1D<R, C, NTH> w;  // the stage's working arrays (as the per-stage kernel)
   // float-pair averages (COMP): low parts of the stage input's averages (sm.u
   // slots) and the flux increments f(hi_{e+1}) - f(hi_e) (sm.fm slots)
   R ulo[COMP ? C : 1][COMP ? NTH : 1];
   R fb[COMP ? C : 1][COMP ? NTH : 1];
+  // CL: the halo as the neighbours push it and every warp's maximum wave speed
+  // (bits), by stage parity; this CTA's own first and last three cells
+  float mbox[CL ? 2 : 1][CL ? 6 : 1][CL ? C * NV : 1];
+  float pub[CL ? 6 : 1][CL ? C * NV : 1];
+  unsigned ent[CL ? 2 : 1][CL ? kMaxCluster * (NTH / 32) : 1];
   int abort;            // a wait ran out: every thread leaves
   unsigned red_max[2];  // the CTA's maximum wave speed (bits), per stage parity
   unsigned arrived[2];  // warps that have folded theirs in
   unsigned trb;         // troubled cell-stages of the run
 };
 
-template <typename R, int C, int NTH, bool COMP>
-__global__ void __launch_bounds__(NTH + 32, NTH == 256 ? 2 : 1) resident1d_kernel(Resident1DArgs r) {
+// The address of a shared-memory variable of this CTA in CTA `rank` of the cluster,
+// and a store to it.
+__device__ __forceinline__ void st_cluster(const void* mine, int rank, unsigned v) {
+  unsigned a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(mine)), "r"(rank));
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+// Every thread of every CTA of the run meets (a single CTA: of the CTA).
+__device__ __forceinline__ void cluster_meet(int ncta) {
+  __syncwarp();
+  if (ncta == 1) {
+    asm volatile("bar.sync 0;" ::: "memory");
+  } else {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+}
+
+template <typename R, int C, int NTH, bool COMP, bool CL>
+__global__ void __launch_bounds__(NTH + 32, NTH == 256 && !CL ? 2 : 1) resident1d_kernel(Resident1DArgs r) {
   static_assert(sizeof(R) == 4, "the exchange words carry FP32 values");
-  __shared__ SmemRes<R, C, NTH, COMP> S;
+  __shared__ SmemRes<R, C, NTH, COMP, CL> S;
   Smem1D<R, C, NTH>& sm = S.w;
   const Stage1DArgs& a = r.a;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -125,8 +156,7 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 ? 2 : 1) resident1d_kerne
   const int base = q * T;
   const int Tq = min(T, n - base);  // this CTA's cells (the last tile may be short)
   u64* const hal = r.halo;                 // [cta][parity][6 slots][C][NV]
-  constexpr int NV = COMP ? 3 : 2;         // words per cell and component: average, first
-                                           // moment (, low part of the average)
+  constexpr int NV = COMP ? 3 : 2;         // words per cell and component
   constexpr int HS = 6 * C * NV;           // values of one CTA's published cells
 
   if (tid == 0) {
@@ -136,6 +166,7 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 ? 2 : 1) resident1d_kerne
     S.trb = 0u;
   }
   __syncthreads();
+  if constexpr (CL) cluster_meet(ncta);  // every CTA runs: its shared memory may be written
 
   if (tid >= NT) {
     // ---- the scalar warp ------------------------------------------------
@@ -171,7 +202,12 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 ? 2 : 1) resident1d_kerne
         // entries and publishes alpha, the others read that one word
         float m = 0.0f;
         bool got;
-        if (q == 0) {
+        if constexpr (CL) {  // every warp's maximum is here: the cluster has met
+          unsigned b = 0u;
+          for (int k = lane; k < ncta * NW; k += 32) b = max(b, S.ent[(s - 1) & 1][k]);
+          m = __uint_as_float(__reduce_max_sync(0xffffffffu, b));
+          got = true;
+        } else if (q == 0) {
           got = gather_max(ent + (size_t)((s - 1) & 1) * ncta * kEntStride, ncta, (unsigned)s,
                            lane, &m, r.polls);
           if (got && lane == 0) st_relaxed(r.alpha_word + ((s - 1) & 1), tagged((unsigned)s, m));
@@ -216,14 +252,24 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 ? 2 : 1) resident1d_kerne
         rem = tf > 0.0 ? tf - t : (double)INFINITY;
         ++done_steps;
       }
+      if constexpr (CL) cluster_meet(ncta);
     }
     // alpha of the final state for the next call (slot 0 of the first
     // buffer, the other slots and the second buffer zero, as the per-stage
     // launches leave them), once every CTA has published its last stage
     if (q == 0 && ok && s_end > 0) {
       float m = 0.0f;
-      if (gather_max(ent + (size_t)((s_end - 1) & 1) * ncta * kEntStride, ncta, (unsigned)s_end,
-                     lane, &m, r.polls)) {
+      bool got;
+      if constexpr (CL) {
+        unsigned b = 0u;
+        for (int k = lane; k < ncta * NW; k += 32) b = max(b, S.ent[(s_end - 1) & 1][k]);
+        m = __uint_as_float(__reduce_max_sync(0xffffffffu, b));
+        got = true;
+      } else {
+        got = gather_max(ent + (size_t)((s_end - 1) & 1) * ncta * kEntStride, ncta, (unsigned)s_end,
+                         lane, &m, r.polls);
+      }
+      if (got) {
         const double am = (double)m;
         double* p0 = static_cast<double*>(r.part0);
         double* p1 = static_cast<double*>(r.part1);
@@ -307,7 +353,19 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 ? 2 : 1) resident1d_kerne
           if constexpr (COMP) S.ulo[c][tid + H] = curl[c];
         }
       }
-      if (hj >= 0) {
+      if constexpr (CL) {
+        if (hj >= 0) {
+          const float* src = hs.cta == q ? S.pub[hs.slot] : S.mbox[(s - 1) & 1][hj];
+          const int e = hj < 3 ? hj : Tq + hj;
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            const R s0 = hs.mirror ? R(mirror_sign(c, 0)) : R(1);
+            sm.u[c][0][e] = R(src[NV * c + 0]) * s0;
+            sm.u[c][1][e] = R(src[NV * c + 1]) * (hs.mirror ? R(mirror_sign(c, 1)) : R(1));
+            if constexpr (COMP) S.ulo[c][e] = R(src[NV * c + 2]) * s0;
+          }
+        }
+      } else if (hj >= 0) {
         const u64* src = hal + ((size_t)hs.cta * 2 + ((s - 1) & 1)) * HS + hs.slot * (C * NV);
         u64 w[C * NV];
 #pragma unroll
@@ -438,7 +496,7 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 ? 2 : 1) resident1d_kerne
             pair_axpby(t1h, t1l, u0c[c][0], u0l[c], t2h, t2l, wh, wl, bh[c], bl[c]);
           }
         }
-      } else {
+      } else if constexpr (!CL) {
         s1d::rhs_parts_of_cell<R, C, NTH>(sm, tid, gas, inv_dx, L0u, Du, L0v, Dv);
       }
     }
@@ -453,9 +511,13 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 ? 2 : 1) resident1d_kerne
     if (own) {
       const int e = tid + H;
       R Uo[C];
+      // CL: alpha is there as soon as the cluster has met, so the right-hand
+      // side is formed with it, as the per-stage launches do
+      if constexpr (CL && !COMP) s1d::rhs_of_cell<R, C, NTH>(sm, tid, gas, alpha, inv_dx, L0u, L0v);
 #pragma unroll
       for (int c = 0; c < C; ++c) {
-        const R Lu = L0u[c] - alpha * Du[c], Lv = L0v[c] - alpha * Dv[c];
+        const R Lu = CL && !COMP ? L0u[c] : L0u[c] - alpha * Du[c];
+        const R Lv = CL && !COMP ? L0v[c] : L0v[c] - alpha * Dv[c];
         const R wu = sm.u[c][0][e];
         const R wv = (a.variant & HWENO_VARIANT_RAW_COMBINE) ? sm.u[c][1][e] : sm.vl[c][e - 1];
         const R su = wu + dt * Lu, sv = wv + dt * Lv;
@@ -488,7 +550,29 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 ? 2 : 1) resident1d_kerne
       }
       // publish the first and last three cells (the neighbours' halo)
       const int pslot = tid < 3 ? tid : (tid >= Tq - 3 ? 3 + tid - (Tq - 3) : -1);
-      if (pslot >= 0) {
+      if constexpr (CL) {
+        if (pslot >= 0) {
+          float v[C * NV];
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            v[NV * c + 0] = float(cur[c][0]);
+            v[NV * c + 1] = float(cur[c][1]);
+            if constexpr (COMP) v[NV * c + 2] = float(curl[c]);
+          }
+          // the first three go to the left neighbour's right halo, the last three
+          // to the right neighbour's left one (none beyond an end of the domain
+          // that does not wrap: the CTA's own ghosts are read from pub)
+          int to = pslot < 3 ? q - 1 : q + 1;
+          if (a.bc == 0) to = to < 0 ? ncta - 1 : (to == ncta ? 0 : to);
+          const int slot = pslot < 3 ? pslot + 3 : pslot - 3;
+#pragma unroll
+          for (int j = 0; j < C * NV; ++j) {
+            S.pub[pslot][j] = v[j];
+            if (to >= 0 && to < ncta && to != q)
+              st_cluster(&S.mbox[s & 1][slot][j], to, __float_as_uint(v[j]));
+          }
+        }
+      } else if (pslot >= 0) {
         u64* dst = hal + ((size_t)q * 2 + (s & 1)) * HS + pslot * (C * NV);
 #pragma unroll
         for (int c = 0; c < C; ++c) {
@@ -504,7 +588,14 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 ? 2 : 1) resident1d_kerne
     // stage's first barrier orders the shared memory)
     const unsigned wm = __reduce_max_sync(0xffffffffu, __float_as_uint((float)speed));
     const int wc = __popc(__ballot_sync(0xffffffffu, myflag));
-    if (lane == 0) {
+    if constexpr (CL) {
+      if (lane < ncta) {
+        if (ncta == 1) S.ent[s & 1][tid >> 5] = wm;
+        else st_cluster(&S.ent[s & 1][q * NW + (tid >> 5)], lane, wm);
+      }
+      if (lane == 0 && wc) atomicAdd(&S.trb, (unsigned)wc);
+      cluster_meet(ncta);
+    } else if (lane == 0) {
       const int g = s & 1;
       atomicMax(&S.red_max[g], wm);
       if (wc) atomicAdd(&S.trb, (unsigned)wc);
@@ -538,14 +629,14 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 ? 2 : 1) resident1d_kerne
 template <typename R, int C, int NTH, bool COMP>
 cudaError_t resident_occupancy(int* per_sm) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      per_sm, resident1d_kernel<R, C, NTH, COMP>, NTH + 32, 0);
+      per_sm, resident1d_kernel<R, C, NTH, COMP, false>, NTH + 32, 0);
 }
 
 template <typename R, int C, int NTH, bool COMP>
 cudaError_t resident_launch(const Resident1DArgs& r, int ncta, cudaStream_t s) {
   Resident1DArgs rc = r;
   void* args[] = {&rc};
-  return cudaLaunchCooperativeKernel((const void*)resident1d_kernel<R, C, NTH, COMP>, dim3(ncta),
+  return cudaLaunchCooperativeKernel((const void*)resident1d_kernel<R, C, NTH, COMP, false>, dim3(ncta),
                                      dim3(NTH + 32), args, 0, s);
 }
 
@@ -565,6 +656,36 @@ cudaError_t resident_dispatch(int system, int nth, bool comp, const Resident1DAr
                        : resident_c<float, 3, true>(nth, r, ncta, s, per);
   return system == 0 ? resident_c<float, 1, false>(nth, r, ncta, s, per)
                      : resident_c<float, 3, false>(nth, r, ncta, s, per);
+}
+
+// The cluster run: a launch of ncta CTAs that are one cluster (r), or how many
+// such clusters the device holds at once (r = nullptr, *active).
+constexpr int kClusterNth = 256;
+template <int C, bool COMP>
+cudaError_t cluster_c(const Resident1DArgs* r, int ncta, cudaStream_t s, int* active) {
+  auto* kernel = resident1d_kernel<float, C, kClusterNth, COMP, true>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)ncta);
+  cfg.blockDim = dim3(kClusterNth + 32);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)ncta;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaSuccess;
+  if (ncta > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  if (r) return cudaLaunchKernelEx(&cfg, kernel, *r);
+  return cudaOccupancyMaxActiveClusters(active, kernel, &cfg);
+}
+
+cudaError_t cluster_dispatch(int system, bool comp, const Resident1DArgs* r, int ncta, cudaStream_t s,
+                             int* active) {
+  if (system == 0)
+    return comp ? cluster_c<1, true>(r, ncta, s, active) : cluster_c<1, false>(r, ncta, s, active);
+  return comp ? cluster_c<3, true>(r, ncta, s, active) : cluster_c<3, false>(r, ncta, s, active);
 }
 
 // HWENO_FP32C state conversions: an FP64 state [C][M][n] (M moments, n cells)
@@ -655,6 +776,37 @@ cudaError_t launch_resident1d(const Resident1DArgs& r, int nth, int ncta, cudaSt
     e = cudaMemsetAsync(r.entries, 0, sizeof(unsigned long long) * resident1d_entry_words(ncta), s);
   if (e != cudaSuccess) return e;
   return resident_dispatch(r.a.system, nth, r.lo != nullptr, &r, ncta, s, nullptr);
+}
+
+cudaError_t cluster1d_geometry(int system, bool comp, int n, int* tile, int* ncta) {
+  *tile = *ncta = 0;
+  if (n < 6) return cudaSuccess;
+  // one CTA, or equal tiles of about 122 cells (one warp per SM sub-partition) up
+  // to 8 CTAs, the portable cluster size, then of up to 250 cells; every tile (the
+  // last one too) at least 6 cells.  Lax data, us per stage with tiles of up to
+  // 250 / 122 / 58 cells: 200 cells 2.27 / 2.38 / 2.40, 400 cells 2.53 / 2.42 /
+  // 2.45, 800 cells 2.57 / 2.48 / 2.48
+  const int full = kClusterNth - 6;
+  int c0 = (n + full - 1) / full;
+  if (n > full) c0 = std::max(c0, std::min(8, (n + 121) / 122));
+  for (int c = c0; c <= kMaxCluster; ++c) {
+    const int t = (n + c - 1) / c;
+    if ((n + t - 1) / t != c || n - (c - 1) * t < 6) continue;
+    int active = 0;
+    const cudaError_t e = cluster_dispatch(system, comp, nullptr, c, nullptr, &active);
+    if (e != cudaSuccess || active < 1) {
+      cudaGetLastError();  // not on this device: the other launches
+      return cudaSuccess;
+    }
+    *tile = t;
+    *ncta = c;
+    return cudaSuccess;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_cluster1d(const Resident1DArgs& r, int ncta, cudaStream_t s) {
+  return cluster_dispatch(r.a.system, r.lo != nullptr, &r, ncta, s, nullptr);
 }
 
 }  // namespace hw

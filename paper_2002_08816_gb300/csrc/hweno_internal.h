@@ -189,8 +189,8 @@ cudaError_t launch_stage1d(const Stage1DArgs& a, cudaStream_t s);
 // on a small grid takes 26-cell tiles (nth = 32): an SM's FP64 pipe is the
 // bound, so the work goes to as many SMs as there are (200 cells, Lax data: the
 // call 79 us on one 250-cell tile with a cell per thread, 42 us on 26-cell
-// ones); from 304 such
-// tiles (two per SM) on, the larger tiles fill the SMs as well.
+// ones); from 304 such tiles (two per SM) on, the larger tiles fill the SMs as
+// well.
 inline void rhs_tiles1d(Stage1DArgs& a) {
   if (a.fp64 && a.n <= 26 * 304) {
     a.nth = 32;
@@ -252,6 +252,12 @@ cudaError_t launch_join_pairs(const void* hi, const float* lo, double* out, int 
                               cudaStream_t s);
 // Zeroes the exchange words, then launches.
 cudaError_t launch_resident1d(const Resident1DArgs& r, int nth, int ncta, cudaStream_t s);
+
+// The resident run of a small grid (FP32, HWENO_FP32C): its CTAs are one
+// thread-block cluster, or a single CTA, and exchange through shared memory; its
+// tile and CTAs (*tile = 0: too many cells, or no such cluster on this device).
+cudaError_t cluster1d_geometry(int system, bool comp, int n, int* tile, int* ncta);
+cudaError_t launch_cluster1d(const Resident1DArgs& r, int ncta, cudaStream_t s);
 
 // The resident run in FP64 (hweno1d_resident64.cu; single instance, up to
 // two CTAs per SM): its tile and CTAs for n cells (*tile = 0 when the grid does not fit on
