@@ -230,28 +230,17 @@ hweno_status hweno_backward(hweno_handle h, const void* grad_out, void* grad_in,
 hweno_status hweno_rhs_vjp(hweno_handle h, const void* in, const uint8_t* flags, double alpha_x,
                            double alpha_y, const void* lam, void* grad);
 
-/* Chooses how a 1D handle (single instance or batch) runs its steps: per-
- * stage launches captured in CUDA graphs, or one persistent cooperative
- * launch per hweno_step call (every CTA walks its tiles of a stage, then the
- * grid meets at a barrier whose wait is bounded), each with 128, 256 or 512
- * threads per CTA (a tile is that number minus 6 cells), and, for FP32
- * single-instance handles whose tiles fit on the GPU at once, one resident
- * launch per hweno_step call with 256 or 512 threads per CTA (every CTA keeps
- * its tile in shared memory for the whole run and exchanges only 3-cell halos
- * and its maximum wave speed with the others, all waits bounded).  Each
- * candidate advances the current state nsteps_trial steps once untimed (which
- * builds its graphs) and then twice timed with CUDA events on the handle's
- * stream; the one with the fastest trial is kept for later calls; the
- * state, time, counters and wave-speed slots are restored afterwards.  The
- * per-stage candidates give bitwise the same results; the persistent and
- * resident ones agree with them to rounding (their copy of the stage body may
- * contract a few multiply-adds differently).  The paper has no counterpart (it
- * fixes no hardware mapping).  choice_out (nullable, 2 ints) receives the
- * threads per CTA and the launch kind (0 graphs, 1 persistent, 2 resident).
- * New handles start with 256 threads and per-stage graphs (HWENO_FP32C: the
- * resident launch, the only one it has; its autotuner times 256 and 512
- * threads).  Waits for the stream; HWENO_ERR_ARG for 2D handles,
- * HWENO_ERR_STATE before set_state. */
+/* Chooses how a 1D handle (single instance or batch) runs its steps among the
+ * choices of hweno_set_execution.  Each candidate advances the current state
+ * nsteps_trial steps once untimed (which builds its graphs) and then twice
+ * timed with CUDA events on the handle's stream; the one with the fastest trial
+ * is kept for later calls; the state, time, counters and wave-speed slots are
+ * restored afterwards.  The paper has no counterpart (it fixes no hardware
+ * mapping).  choice_out (nullable, 2 ints) receives the threads per CTA and the
+ * launch kind (0 graphs, 1 persistent, 2 resident).  New handles start with 256
+ * threads and kind 0 (HWENO_FP32C: kind 2, the only one it has; its autotuner
+ * times 256 and 512 threads).  Waits for the stream; HWENO_ERR_ARG for 2D
+ * handles, HWENO_ERR_STATE before set_state. */
 hweno_status hweno_autotune(hweno_handle h, int nsteps_trial, int* choice_out);
 
 /* Failure-detection self-test of the grid barrier the persistent launch uses
@@ -285,13 +274,21 @@ hweno_status hweno_check_resident(hweno_handle h, int nsteps, int silent_cta, un
 
 /* Sets the choice hweno_autotune makes by hand: threads per CTA (128, 256 or
  * 512) and the launch kind: 0 per-stage launches in CUDA graphs, 1 one
- * persistent launch per hweno_step with a grid barrier between stages, 2 one
- * resident launch per hweno_step in which every CTA keeps its tile of the
- * state in shared memory for the whole run (FP32 single-instance handles, 256
- * or 512 threads, grids small enough for every tile to be on the GPU at once;
- * HWENO_ERR_ARG otherwise; HWENO_FP32C handles take only this kind).  1D
- * handles only; waits for the stream.  All choices compute the same scheme;
- * results agree to rounding (the per-stage choices bit for bit). */
+ * persistent launch per hweno_step with a grid barrier between stages (FP64; an
+ * FP32 handle runs its per-stage launches), 2 one resident launch per
+ * hweno_step in which every CTA keeps its tile of the state in shared memory
+ * for the whole run (FP32 single-instance handles, 256 or 512 threads, grids
+ * small enough for every tile to be on the GPU at once; HWENO_ERR_ARG
+ * otherwise; HWENO_FP32C handles take only this kind).
+ * A single instance whose tiles fit on the GPU at once runs resident under every
+ * choice, because nothing else is as fast there: grids of 6 to about 4000 cells
+ * in FP32 and HWENO_FP32C as one thread-block cluster, up to about 76000 cells
+ * in FP32 and FP64 as one cooperative launch.  The choice then selects among
+ * the launches of batches, larger grids and grids below 6 cells, and with kind 2
+ * the resident launch's threads; a single FP32 instance's stage launches take
+ * their threads from its size.  1D handles only; waits for the stream.  All
+ * choices compute the same scheme; results agree to rounding (kinds 0 with
+ * different threads bit for bit). */
 hweno_status hweno_set_execution(hweno_handle h, int threads, int persistent);
 
 /* The conserved totals of the current state: totals[c] = the sum over cells

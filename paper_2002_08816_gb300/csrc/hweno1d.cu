@@ -1,52 +1,47 @@
 // The 1D kernels: one launch per third-order TVD Runge-Kutta stage (captured
-// in CUDA graphs by the C ABI, with programmatic dependent launch), or a whole
-// run in one persistent cooperative launch; both inline the same stage body
-// (hweno1d_stage.cuh).  Also the wave-speed kernels that start a
-// run and small helpers (conversions, device scalars).
+// in CUDA graphs by the C ABI, with programmatic dependent launch), or, in FP64,
+// a whole run in one persistent cooperative launch; the stage bodies are those
+// of hweno1d_pair.cuh (FP32) and hweno1d_stage64.cuh (FP64).  Also the
+// wave-speed kernels that start a run and small helpers (conversions, device
+// scalars).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "hweno1d_pair.cuh"
 #include "hweno1d_stage64.cuh"
 
 namespace hw {
 namespace {
 
 using s1d::H;
-using s1d::Smem1D;
 using s1d::wave_speed;
 constexpr int NT = kThreads1D;  // threads of the wave-speed kernels
 constexpr int T = kTile1D;      // their cells per CTA
 constexpr int NW = NT / 32;
 
 // Every CTA has NTH cell threads and one scalar warp (hweno1d_stage.cuh).
-// FP32: a tile is NTH - 6 cells, a cell per thread; the 128-thread tiles are
-// the high-occupancy choice (8 CTAs per SM, at most 51 registers), which hides
-// the stage's dependent load and arithmetic chains on large states and
-// batches; on small states, which sit at the per-stage latency floor, the
-// 256-thread tiles at the register count the compiler picks are faster.
-// hweno_autotune chooses.  FP64: the tasks of hweno1d_fp64.cuh on the same
-// tiles, and on tiles of 26 cells with 128 threads (nth = 32, stage_nth) for
-// grids that leave SMs idle otherwise.
-template <typename R, int NTH>
-constexpr int tile_cells() { return NTH == 32 ? 26 : NTH - 2 * H; }
+// FP32: two cells per thread in packed FP32 (hweno1d_pair.cuh), tiles of 2 NTH -
+// 12 cells.  FP64: the tasks of hweno1d_fp64.cuh on tiles of NTH - 6 cells, and
+// on tiles of 26 cells with 128 threads (nth = 32, rhs_tiles1d) for grids that
+// leave SMs idle otherwise.  stage1d_cells gives a tile's cells on the host.
 template <typename R, int NTH>
 constexpr int cell_threads() { return NTH == 32 ? 128 : NTH; }
 template <typename R, int NTH>
 constexpr int min_ctas() {
-  return sizeof(R) == 4 ? (NTH == 128 ? 8 : 1) : (NTH <= 128 ? 4 : NTH == 256 ? 2 : 1);
+  return sizeof(R) == 4 ? (NTH == 128 ? 5 : NTH == 256 ? 2 : 1) : (NTH <= 128 ? 4 : NTH == 256 ? 2 : 1);
 }
 
 // One tile of one stage; the tile's arrays are in dynamic shared memory.
 template <typename R, int C, bool BATCH, int NTH>
 struct StageTile {
-  typedef Smem1D<R, C, NTH> Smem;
+  typedef pr::SmemPair<C, NTH> Smem;
   static __device__ __forceinline__ void run(const Stage1DArgs& a, int tile, Smem& sm) {
-    s1d::stage1d_tile<R, C, BATCH, NTH>(a, tile, sm);
+    pr::stage_tile<C, BATCH, NTH>(a, tile, sm);
   }
 };
 template <int C, bool BATCH, int NTH>
 struct StageTile<double, C, BATCH, NTH> {
-  static constexpr int T = tile_cells<double, NTH>(), N = cell_threads<double, NTH>();
+  static constexpr int T = NTH == 32 ? 26 : NTH - 2 * H, N = cell_threads<double, NTH>();
   typedef f64::Smem64<C, T> Smem;
   static __device__ __forceinline__ void run(const Stage1DArgs& a, int tile, Smem& sm) {
     f64::stage64_tile<C, BATCH, T, N>(a, tile, sm);
@@ -62,8 +57,8 @@ __global__ void __launch_bounds__(cell_threads<R, NTH>() + 32, min_ctas<R, NTH>(
 }
 
 // ------------------------------------------------------------ persistent run
-// A whole run of Runge-Kutta steps in one cooperative launch: each CTA applies
-// the stage body to its tiles of a stage, then all CTAs meet at a grid barrier
+// A whole run of Runge-Kutta steps in one cooperative launch (FP64 batches and
+// grids too large for the resident run): each CTA applies the stage body to its tiles of a stage, then all CTAs meet at a grid barrier
 // before the next stage reads their outputs and the alpha slots they filled.
 // The barrier's wait is bounded: after kBarrierPolls polls (about a second)
 // the CTA sets ST_TIMEOUT in the status word and returns, and the others give
@@ -196,7 +191,7 @@ cudaError_t run_b(const Run1DArgs& r, cudaStream_t s) {
 
 template <typename R, int C>
 cudaError_t run_c(const Run1DArgs& r, cudaStream_t s) {
-  return r.a.tile_inst ? run_b<R, C, true>(r, s) : run_b<R, C, false>(r, s);
+  return r.a.btile ? run_b<R, C, true>(r, s) : run_b<R, C, false>(r, s);
 }
 
 // Wave-speed maxima in FP64 slots (the per-cell speeds in the kernel's
@@ -230,26 +225,22 @@ __global__ void __launch_bounds__(NT) alpha1d_kernel(const R* __restrict__ w, do
 }
 
 // Wave-speed maxima of every instance of a batch, one slot per instance (the
-// batch's tiles: NTH threads, NTH - 6 cells).
-template <typename R, int C, int NTH>
-__global__ void __launch_bounds__(NTH) alpha1d_batch_kernel(Stage1DArgs a) {
-  constexpr int T = NTH - 2 * H, NW = NTH / 32;
+// batch's tiles, of T cells).
+template <typename R, int C>
+__global__ void __launch_bounds__(NT) alpha1d_batch_kernel(Stage1DArgs a, int T) {
   __shared__ R red[NW];
-  const int inst = a.tile_inst[blockIdx.x];
-  const BatchInst& bi = a.binst[inst];
-  const int i = a.tile_base[blockIdx.x] + threadIdx.x;
+  const BatchTile& bi = a.btile[blockIdx.x];
+  const int inst = bi.inst;
   const R* w = static_cast<const R*>(a.w) + bi.off;
-  const int n = bi.n;
+  const int n = bi.n, end = min(bi.base + T, n);
   R s = R(0);
-  if (threadIdx.x < T && i < n) {
+  for (int i = bi.base + threadIdx.x; i < end; i += NT) {
     R U[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) U[c] = w[(2 * c) * n + i];
-    s = wave_speed<R, C>(R(a.gas), U);
-    if (!(s == s)) {
-      atomicOr(&a.sc->status, (unsigned)ST_NONPHYSICAL);
-      s = R(0);
-    }
+    const R v = wave_speed<R, C>(R(a.gas), U);
+    if (v == v) s = fmax(s, v);
+    else atomicOr(&a.sc->status, (unsigned)ST_NONPHYSICAL);
   }
   for (int o = 16; o > 0; o >>= 1) s = fmax(s, __shfl_xor_sync(0xffffffffu, s, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
@@ -361,21 +352,18 @@ cudaError_t launch_stage1d_b(const Stage1DArgs& a, cudaStream_t s) {
 
 template <typename R, int C>
 cudaError_t launch_stage1d_t(const Stage1DArgs& a, cudaStream_t s) {
-  return a.tile_inst ? launch_stage1d_b<R, C, true>(a, s) : launch_stage1d_b<R, C, false>(a, s);
+  return a.btile ? launch_stage1d_b<R, C, true>(a, s) : launch_stage1d_b<R, C, false>(a, s);
 }
 
 template <typename R, int C>
 void alpha1d_batch_t(const Stage1DArgs& a, cudaStream_t s) {
-  if (a.nth == 128) alpha1d_batch_kernel<R, C, 128><<<a.ntile, 128, 0, s>>>(a);
-  else if (a.nth == 512) alpha1d_batch_kernel<R, C, 512><<<a.ntile, 512, 0, s>>>(a);
-  else alpha1d_batch_kernel<R, C, 256><<<a.ntile, 256, 0, s>>>(a);
+  alpha1d_batch_kernel<R, C><<<a.ntile, NT, 0, s>>>(a, stage1d_cells(a.fp64, a.nth));
 }
 
 }  // namespace
 
 cudaError_t launch_run1d(const Run1DArgs& r, cudaStream_t s) {
-  if (r.a.system == 0) return r.a.fp64 ? run_c<double, 1>(r, s) : run_c<float, 1>(r, s);
-  return r.a.fp64 ? run_c<double, 3>(r, s) : run_c<float, 3>(r, s);
+  return r.a.system == 0 ? run_c<double, 1>(r, s) : run_c<double, 3>(r, s);
 }
 
 cudaError_t launch_barrier_check(int ctas, int meetings, int missing, unsigned polls,

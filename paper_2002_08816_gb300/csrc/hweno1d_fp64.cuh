@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "hweno1d_fields.cuh"
 #include "hweno1d_stage.cuh"
 
 namespace hw {
@@ -106,143 +107,6 @@ __device__ __forceinline__ void flux(double gas, const double* U, double* F) {
   }
 }
 
-// One characteristic field of the Jacobian at U: left eigenvector row l, right
-// eigenvector column r (Burgers: the identity).
-template <int C>
-__device__ __forceinline__ void field(double gas, const double* U, int f, double* l, double* r) {
-  if constexpr (C == 1) {
-    l[0] = r[0] = 1.0;
-  } else {
-    const double ir = __drcp_rn(U[0]), mu = U[1] * ir;
-    const double mu2 = mu * mu;
-    const double p = (gas - 1.0) * fma(-0.5 * U[0], mu2, U[2]);
-    const double c = sqrt(gas * p * ir);
-    const double ic = __drcp_rn(c);
-    const double b1 = (gas - 1.0) * ic * ic, b2 = 0.5 * b1 * mu2;
-    if (f == 1) {
-      l[0] = 1.0 - b2; l[1] = b1 * mu; l[2] = -b1;
-      r[0] = 1.0; r[1] = mu; r[2] = 0.5 * mu2;
-    } else {
-      const double s = f == 0 ? 1.0 : -1.0;  // mu - c, mu + c
-      const double H = (U[2] + p) * ir;
-      l[0] = 0.5 * fma(s * mu, ic, b2);
-      l[1] = -0.5 * fma(b1, mu, s * ic);
-      l[2] = 0.5 * b1;
-      r[0] = 1.0; r[1] = fma(-s, c, mu); r[2] = fma(-s * mu, c, H);
-    }
-  }
-}
-
-// Sum over a cell's fields of r_f[c] x_f, for component c = this lane's own
-// place among the cell's C lanes (base: the first of them).
-template <int C>
-__device__ __forceinline__ double to_component(const double* r, double x, int f, int base) {
-  if constexpr (C == 1) {
-    return x;
-  } else {
-    double t[C], mine[C];
-#pragma unroll
-    for (int c = 0; c < C; ++c) t[c] = r[c] * x;
-#pragma unroll
-    for (int g = 0; g < C; ++g) {
-#pragma unroll
-      for (int c = 0; c < C; ++c) {
-        const double v = __shfl_sync(0xffffffffu, t[c], base + g);
-        if (c == f) mine[g] = v;
-      }
-    }
-    return mine[0] + mine[1] + mine[2];
-  }
-}
-
-// Weights3's combination, with reciprocals (5.4 FP64 instructions each against
-// 8.5 for a quotient) and w_0 / gamma_0 formed without the division by gamma_0.
-struct Weights {
-  double w0g, w1, w2, g1, g2;
-  __device__ __forceinline__ Weights(const double* gam, double eps, double b0, double b1, double b2) {
-    const double s = 0.5 * (fabs(b0 - b1) + fabs(b0 - b2));
-    const double tau = s * s;
-    const double a0 = fma(tau, __drcp_rn(b0 + eps), 1.0);
-    const double a1 = gam[1] * fma(tau, __drcp_rn(b1 + eps), 1.0);
-    const double a2 = gam[2] * fma(tau, __drcp_rn(b2 + eps), 1.0);
-    const double inv = __drcp_rn(fma(gam[0], a0, a1) + a2);
-    w0g = a0 * inv;
-    w1 = a1 * inv;
-    w2 = a2 * inv;
-    g1 = gam[1];
-    g2 = gam[2];
-  }
-  __device__ __forceinline__ double apply(double v0, double v1, double v2) const {
-    return fma(w0g, fma(-g2, v2, fma(-g1, v1, v0)), fma(w1, v1, w2 * v2));
-  }
-};
-
-// The smoothness indicators of the high-degree candidates of Step 1 and Step
-// 2.1 as sums of 4 and 5 squares instead of the printed 5 and 8: each is a
-// quadratic form without terms mixing the even data (c = u_m - 2 u_0 + u_p, dV
-// = v_m - v_p) and the odd ones (dU = u_m - u_p, sV = v_m + v_p, v_0), so an
-// exact LDL^T of the two blocks gives it in 10 and 14 operations (the printed
-// forms 20 and 37); the even block is the same in both.  Every term is
-// positive, and dU^2 and c^2 carry the energy of smooth data.
-__device__ __forceinline__ double even_beta(double c, double dV) {
-  const double s = fma(110741.0 / 660750.0, c, dV);
-  return fma((1421461.0 / 1321500.0) * c, c, ((991125.0 / 112.0) * s) * s);
-}
-
-// Step 1 of one field: the modified first moment.
-__device__ __forceinline__ double limit_moment(double um, double u0, double up, double vm, double vp,
-                                               const double* gam, double eps) {
-  const double d1 = u0 - um, d2 = up - u0, dU = um - up, sV = vm + vp, dV = vm - vp;
-  const double cU = d2 - d1;  // u_m - 2 u_0 + u_p
-  const double s = fma(839.0 / 9612.0, dU, sV);
-  const double b0 = fma((781.0 / 3204.0) * dU, dU, fma((144180.0 / 361.0) * s, s, even_beta(cU, dV)));
-  const Weights w(gam, eps, b0, d1 * d1, d2 * d2);
-  return w.apply(fma(-5.0 / 76.0, dU, (-11.0 / 38.0) * sV), (1.0 / 12.0) * d1, (1.0 / 12.0) * d2);
-}
-
-// p0 by its even and odd parts about x_i: the faces (Step 2.2), and the interior
-// Gauss-Lobatto points (Step 2.3), as u_0 plus an increment (the coefficients
-// of the averages sum to one), so that each value is rounded once at the size
-// of u: two mirror images that shared a rounded even part would carry the
-// same error into both moment equations (smooth density wave, 40 steps, error
-// against 80 bits: shared 2.4e-15, plain sums of six terms 1.8e-15).  D = u_p -
-// u_m, c = u_m - 2 u_0 + u_p, sV = v_m + v_p, dV = v_m - v_p.
-__device__ __forceinline__ void p0_faces(double u0, double D, double c, double sV, double dV, double v0,
-                                         double& left, double& right) {
-  const double even = fma(5.0 / 24.0, c, 0.75 * dV);
-  const double odd = fma(19.0 / 216.0, D, fma(-31.0 / 108.0, sV, (241.0 / 54.0) * v0));
-  left = u0 + (even - odd);
-  right = u0 + (even + odd);
-}
-__device__ __forceinline__ void p0_interior(double u0, double D, double c, double sV, double dV,
-                                            double v0, double& gm, double& gp) {
-  constexpr double r5 = 2.2360679774997896964;
-  const double even = fma(-1.0 / 24.0, c, -0.15 * dV);
-  const double odd = fma(-101.0 / 5400.0 * r5, D, fma(841.0 / 13500.0 * r5, sV, (10289.0 / 6750.0 * r5) * v0));
-  gm = u0 + (even - odd);
-  gp = u0 + (even + odd);
-}
-
-// Step 2.1 of one field: the HWENO values at both interfaces.
-__device__ __forceinline__ void hweno(double um, double u0, double up, double vm, double v0, double vp,
-                                      const double* gam, double eps, double& left, double& right) {
-  const double d1 = u0 - um, d2 = up - u0, dU = um - up, sV = vm + vp, dV = vm - vp;
-  const double cU = d2 - d1;  // u_m - 2 u_0 + u_p
-  double p0l, p0r;
-  p0_faces(u0, -dU, cU, sV, dV, v0, p0l, p0r);
-  const double h1 = fma(1.0 / 6.0, um, (5.0 / 6.0) * u0), h2 = fma(1.0 / 6.0, up, (5.0 / 6.0) * u0);
-  const double s = fma(23124050207.0 / 264871203420.0, dU, sV);
-  const double r = fma(2632162559.0 / 40053970660.0, dU, fma(1155959005.0 / 4005397066.0, sV, v0));
-  const double b0 = fma((21520059541.0 / 88290401140.0) * dU, dU,
-                    fma((794613610260.0 / 2002698533.0) * s, s,
-                    fma((10013492665.0 / 2916.0) * r, r, even_beta(cU, dV))));
-  const double v2 = (144.0 * v0) * v0;
-  const double e1 = fma(12.0, v0, -d1), e2 = fma(12.0, v0, -d2);
-  const Weights w(gam, eps, b0, fma((13.0 / 3.0) * e1, e1, v2), fma((13.0 / 3.0) * e2, e2, v2));
-  left = w.apply(p0l, fma(-4.0, v0, h1), fma(-8.0, v0, h2));
-  right = w.apply(p0r, fma(8.0, v0, h1), fma(4.0, v0, h2));
-}
-
 // The parameters of a stage.
 struct Par {
   double gam[3], eps, gas, h, thr, inv_dx;
@@ -292,7 +156,7 @@ __device__ __forceinline__ int step1(Smem64<C, TMAX>& sm, const double (*u)[2][T
       double U[C], l[C], r[C], d[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll
       for (int c = 0; c < C; ++c) U[c] = u[c][0][e];
-      field<C>(a.gas, U, f, l, r);
+      fld::field<double, C>(a.gas, U, f, l, r);
 #pragma unroll
       for (int c = 0; c < C; ++c) {
         d[0] = fma(l[c], u[c][0][e - 1], d[0]);
@@ -301,7 +165,7 @@ __device__ __forceinline__ int step1(Smem64<C, TMAX>& sm, const double (*u)[2][T
         d[3] = fma(l[c], u[c][1][e - 1], d[3]);
         d[4] = fma(l[c], u[c][1][e + 1], d[4]);
       }
-      const double v = to_component<C>(r, limit_moment(d[0], d[1], d[2], d[3], d[4], a.gam, a.eps), f,
+      const double v = fld::to_component<double, C>(r, fld::limit_moment(d[0], d[1], d[2], d[3], d[4], a.gam, a.eps), f,
                                        min(base, 32 - C));
       if (on) sm.vl[f][e] = v;
     }
@@ -324,8 +188,8 @@ __device__ __forceinline__ void step2(Smem64<C, TMAX>& sm, const double (*u)[2][
     const double d1 = u0 - um, d2 = up - u0, sV = vm + vp, dV = vm - vp;
     const double D = d2 + d1, cU = d2 - d1;
     double l, r, gm, gp;
-    p0_faces(u0, D, cU, sV, dV, v0, l, r);
-    p0_interior(u0, D, cU, sV, dV, v0, gm, gp);
+    fld::p0_faces(u0, D, cU, sV, dV, v0, l, r);
+    fld::p0_interior(u0, D, cU, sV, dV, v0, gm, gp);
     sm.P[0][c][e] = l;
     sm.P[1][c][e] = r;
     sm.P[2][c][e] = gm;
@@ -346,7 +210,7 @@ __device__ __forceinline__ void step2(Smem64<C, TMAX>& sm, const double (*u)[2][
 #pragma unroll
         for (int c = 0; c < C; ++c)
           B[c] = mean ? 0.5 * (u[c][0][e - 1 + side] + u[c][0][e + side]) : u[c][0][e];
-        field<C>(a.gas, B, f, l, r);
+        fld::field<double, C>(a.gas, B, f, l, r);
 #pragma unroll
         for (int c = 0; c < C; ++c)
 #pragma unroll
@@ -355,14 +219,14 @@ __device__ __forceinline__ void step2(Smem64<C, TMAX>& sm, const double (*u)[2][
             d[3 + j] = fma(l[c], sm.vl[c][e - 1 + j], d[3 + j]);
           }
         double cl, cr;
-        hweno(d[0], d[1], d[2], d[3], d[4], d[5], a.gam, a.eps, cl, cr);
+        fld::hweno(d[0], d[1], d[2], d[3], d[4], d[5], a.gam, a.eps, cl, cr);
         const int b = min(base, 32 - C);
         if (!mean || side == 0) {
-          const double v = to_component<C>(r, cl, f, b);
+          const double v = fld::to_component<double, C>(r, cl, f, b);
           if (on) sm.P[0][f][e] = v;
         }
         if (!mean || side == 1) {
-          const double v = to_component<C>(r, cr, f, b);
+          const double v = fld::to_component<double, C>(r, cr, f, b);
           if (on) sm.P[1][f][e] = v;
         }
       }

@@ -1,34 +1,32 @@
-// The body of one third-order TVD Runge-Kutta stage of the 1D hybrid HWENO
-// scheme (Zhao & Qiu, arXiv:2002.08816, Sec. 2.1) on one tile, shared by the
-// per-stage kernel and the persistent kernel (hweno1d.cu).
+// What the 1D kernels of the hybrid HWENO scheme share (Zhao & Qiu,
+// arXiv:2002.08816, Sec. 2.1): the scalar warp of a tile, and the phases of one
+// third-order TVD Runge-Kutta stage with a cell per thread, which the resident
+// FP32 runs inline (hweno1d_resident.cu).  The per-stage launches run FP32 with
+// two cells per thread (hweno1d_pair.cuh) and FP64 in tasks (hweno1d_fp64.cuh).
 //
-// A CTA of NTH + 32 threads owns T = NTH - 6 consecutive cells: NTH cell
-// threads and one scalar warp.  The cell threads stage the cells plus a
-// 3-cell halo of the stage input in shared memory (coalesced loads of each
-// structure-of-arrays row), then, all on chip:
+// A CTA has NTH cell threads and one scalar warp.  The cell threads hold the
+// tile's cells and a 3-cell halo of the stage input in shared memory, then, all
+// on chip:
 //   1. (scalar warp, concurrently with steps 2-3 of the cell threads, all in
 //      FP64) alpha = max |f'(ubar)| over the maxima the producer of the stage
-//      input left in kAlphaSlots FP64 slots (global Lax-Friedrichs flux);
-//      stage 1 also turns alpha into dt = CFL dx / alpha, clipped to t_final;
-//      the lead tile records dt and, in stage 3, the time.  The per-cell
-//      wave speeds are bulk arithmetic in the kernel's precision; their
-//      maximum, dt, the clipping and the time are FP64, off the cell
-//      threads' critical path (a dependent FP64 operation costs tens of
-//      cycles on GB300, a division hundreds);
+//      input left (global Lax-Friedrichs flux); stage 1 also turns alpha into
+//      dt = CFL dx / alpha, clipped to t_final; the lead tile records dt and, in
+//      stage 3, the time.  The per-cell wave speeds are bulk arithmetic in the
+//      kernel's precision; their maximum, dt, the clipping and the time are FP64,
+//      off the cell threads' critical path (a dependent FP64 operation costs
+//      tens of cycles on GB300, a division hundreds);
 //   2. KXRCF flags and the modified first moments (Step 1) for the cells and
-//      2 halo cells per side, in characteristic fields for Euler (out-of-line
-//      work of the troubled lanes); an FP32 kernel decides a flag in FP32 when
-//      its rounding-error bound allows and by an error-free float-pair
-//      evaluation otherwise, so flags equal the FP64 decision off the threshold;
+//      2 halo cells per side, in characteristic fields for Euler; an FP32 kernel
+//      decides a flag in FP32 when its rounding-error bound allows and by an
+//      error-free float-pair evaluation otherwise, so flags equal the FP64
+//      decision off the threshold;
 //   3. interface values (Steps 2.1/2.2) for the cells and 1 halo cell per
 //      side: linear p0 unless a cell of S0 = {i-1, i, i+1} is troubled;
 //   4. for the own cells: interior Gauss-Lobatto values (Step 2.3), the
 //      Lax-Friedrichs fluxes at x_{i-+1/2}, F_i, the right-hand sides of
 //      Eq. (odeH) and the Runge-Kutta combination of Eq. (RK);
-//   5. the maximum wave speed of the output, folded by FP64 atomic max into
-//      the tile's one of kAlphaSlots slots that the next stage reads for its alpha
-//      (warp by warp, or after a CTA reduction on large grids), the troubled
-//      count and the status bits (non-finite, non-physical).
+//   5. the maximum wave speed of the output for the next stage's alpha, the
+//      troubled count and the status bits (non-finite, non-physical).
 // The limited stage input is what the RK combination uses (the first moment
 // of a troubled cell is modified in the state, as a DG limiter would).
 #pragma once
@@ -44,8 +42,6 @@ namespace hw {
 namespace s1d {
 
 constexpr int H = 3;  // halo cells per side
-// grids of at most this many tiles fold the wave-speed maxima warp by warp
-constexpr int kWarpAtomicTiles = 2048;
 
 // Named barriers: kBarCells among the NTH cell threads only; kBarAll for the
 // cell threads and the scalar warp (which only arrives) before step 4.
@@ -349,9 +345,9 @@ __device__ __forceinline__ TileAt tile_at(Stage1DArgs& a, int tile, int T) {
   TileAt x = {a.n, tile * T, 0, tile == 0};
   if constexpr (BATCH) {
     // a batch of independent instances: this tile's instance and first cell
-    x.inst = a.tile_inst[tile];
-    x.base = a.tile_base[tile];
-    const BatchInst& bi = a.binst[x.inst];
+    const BatchTile bi = a.btile[tile];
+    x.inst = bi.inst;
+    x.base = bi.base;
     x.n = bi.n;
     x.lead = x.base == 0;
     const long long off = bi.off;
@@ -368,7 +364,6 @@ __device__ __forceinline__ TileAt tile_at(Stage1DArgs& a, int tile, int T) {
     a.hthr = bi.hthr_f;
     a.hthr_lo = bi.hthr_lo_f;
     a.f32[5] = bi.inv_dx_f;
-    a.f32[6] = bi.cfl_dx_f;
   }
   return x;
 }
@@ -472,218 +467,6 @@ __device__ __forceinline__ void scalar_warp(const Stage1DArgs& a, int tile, int 
     }
   }
   bar_arrive(kBarAll, nt + 32);
-}
-
-// One stage on one tile of T = NTH - 6 cells, by a CTA of NTH + 32 threads.  The
-// per-stage kernel calls it once; the persistent kernel calls it for each of
-// its tiles of each stage, between grid barriers, so every load of data
-// produced in the same launch goes through L2 (ldx).
-template <typename R, int C, bool BATCH, int NTH>
-__device__ __forceinline__ void stage1d_tile(Stage1DArgs a, const int tile, Smem1D<R, C, NTH>& sm) {
-  constexpr int T = NTH - 2 * H, NT = NTH, NW = NTH / 32;
-  const int tid = threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
-  const TileAt at = tile_at<R, C, BATCH>(a, tile, T);
-  const int n = at.n, base = at.base, inst = at.inst;
-  const R* __restrict__ w = static_cast<const R*>(a.w);
-
-  // The producer of the stage input may still be finishing (programmatic
-  // dependent launch): wait for its completion and memory before any read.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-
-  // Parameters in the kernel's precision (FP32 copies made on the host).
-  R gam[3], eps, gas, inv_dx;
-  if constexpr (sizeof(R) == 4) {
-    gam[0] = a.f32[0]; gam[1] = a.f32[1]; gam[2] = a.f32[2];
-    eps = a.f32[3]; gas = a.f32[4]; inv_dx = a.f32[5];
-  } else {
-    gam[0] = a.gam[0]; gam[1] = a.gam[1]; gam[2] = a.gam[2];
-    eps = a.eps; gas = a.gas; inv_dx = a.inv_dx;
-  }
-
-  if (tid >= NT) {
-    scalar_warp<R, BATCH>(a, tile, inst, at.lead, lane, NT, &sm.alpha, &sm.dt);
-    return;
-  }
-
-  // ---- the cell threads --------------------------------------------------
-  // 2. in one round trip: the tile-plus-halo element of each thread and, in
-  //    stages 2 and 3, the modified u^n of its own cell
-  R u0c[C][2];
-  if (a.stage >= 2 && tid < T && base + tid < n) {
-    const R* u0 = static_cast<const R*>(a.u0);
-#pragma unroll
-    for (int c = 0; c < C; ++c) {
-      u0c[c][0] = ldx(u0 + (2 * c + 0) * n + base + tid);
-      u0c[c][1] = ldx(u0 + (2 * c + 1) * n + base + tid);
-    }
-  }
-  if (tid < T + 2 * H) {
-    if (a.bc == 2) {
-      bool mir;
-      const int g = bc_map_wall(base - H + tid, n, &mir);
-#pragma unroll
-      for (int c = 0; c < C; ++c) {
-        sm.u[c][0][tid] = ldx(w + (2 * c + 0) * n + g) * (mir ? R(mirror_sign(c, 0)) : R(1));
-        sm.u[c][1][tid] = ldx(w + (2 * c + 1) * n + g) * (mir ? R(mirror_sign(c, 1)) : R(1));
-      }
-    } else {
-      const int g = bc_map(base - H + tid, n, a.bc);
-#pragma unroll
-      for (int c = 0; c < C; ++c) {
-        sm.u[c][0][tid] = ldx(w + (2 * c + 0) * n + g);
-        sm.u[c][1][tid] = ldx(w + (2 * c + 1) * n + g);
-      }
-    }
-  }
-  bar_sync(kBarCells, NT);
-  // the next stage's CTAs may be scheduled now; they wait for this grid above
-  asm volatile("griddepcontrol.launch_dependents;");
-
-  // 3. troubled cells and modified first moments (Step 1), cells base-2 ..
-  //    base+T+1; Euler limits in the characteristic fields of the cell
-  //    average (Remark 2)
-  int flag = 0;
-  if (tid < T + 4) {
-    const int k = tid, e = k + 1;
-    const double h = a.h;
-    const float hthr = a.hthr, hthr_lo = a.hthr_lo;
-    if (a.mode == 1) {
-      flag = 1;
-    } else if (a.mode == 2) {
-      flag = 0;
-    } else if constexpr (C == 1) {
-      const R u0 = sm.u[0][0][e];
-      flag = kxrcf_troubled(sm.u[0][0][e - 1], u0, sm.u[0][0][e + 1], sm.u[0][1][e - 1],
-                            sm.u[0][1][e], sm.u[0][1][e + 1], u0 >= R(0), h, a.thr, hthr, hthr_lo);
-    } else {
-      const bool left = inflow_left(sm.u[0][0][e], sm.u[1][0][e]);
-      flag = kxrcf_troubled(sm.u[0][0][e - 1], sm.u[0][0][e], sm.u[0][0][e + 1],
-                            sm.u[0][1][e - 1], sm.u[0][1][e], sm.u[0][1][e + 1], left, h, a.thr,
-                            hthr, hthr_lo) ||
-             kxrcf_troubled(sm.u[2][0][e - 1], sm.u[2][0][e], sm.u[2][0][e + 1],
-                            sm.u[2][1][e - 1], sm.u[2][1][e], sm.u[2][1][e + 1], left, h, a.thr,
-                            hthr, hthr_lo);
-    }
-    sm.fl[k] = (uint8_t)flag;
-    if (!flag) {
-#pragma unroll
-      for (int c = 0; c < C; ++c) sm.vl[c][k] = sm.u[c][1][e];
-    } else if constexpr (C == 1) {
-      sm.vl[0][k] = limit_first_moment(sm.u[0][0][e - 1], sm.u[0][0][e], sm.u[0][0][e + 1],
-                                       sm.u[0][1][e - 1], sm.u[0][1][e + 1], gam, eps);
-    } else {
-      const ConsVec<R> o = char_limit<R>(
-          gas, gam[0], gam[1], gam[2], eps, sm.u[0][0][e - 1], sm.u[1][0][e - 1],
-          sm.u[2][0][e - 1], sm.u[0][0][e], sm.u[1][0][e], sm.u[2][0][e], sm.u[0][0][e + 1],
-          sm.u[1][0][e + 1], sm.u[2][0][e + 1], sm.u[0][1][e - 1], sm.u[1][1][e - 1],
-          sm.u[2][1][e - 1], sm.u[0][1][e + 1], sm.u[1][1][e + 1], sm.u[2][1][e + 1]);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) sm.vl[c][k] = o.v[c];
-    }
-  }
-  bar_sync(kBarCells, NT);
-
-  // 4. interface values (Steps 2.1, 2.2) and their physical fluxes, cells
-  //    base-1 .. base+T
-  if (tid < T + 2) faces_of_cell<R, C, NTH>(sm, tid, gas, gam, eps, a.variant);
-  // alpha and dt from the scalar warp; a zero dt (t_final reached) is
-  // uniform over the grid (the instance), and the stage then writes nothing
-  bar_sync(kBarAll, NT + 32);
-  const R alpha = sm.alpha, dt = sm.dt;
-  if (a.stage > 0 && !(dt > R(0))) return;
-
-  // 5. own cells: fluxes, F_i, right-hand side, RK combination
-  const int i = base + tid;
-  const bool own = tid < T && i < n;
-  int myflag = 0;
-  R speed = R(0);
-  unsigned bad = 0;
-  if (own) {
-    const int e = tid + H;  // sm.u index
-    myflag = sm.fl[tid + 2];
-    R Lus[C], Lvs[C];
-    rhs_of_cell<R, C, NTH>(sm, tid, gas, alpha, inv_dx, Lus, Lvs);
-    R Uo[C];
-#pragma unroll
-    for (int c = 0; c < C; ++c) {
-      const R Lu = Lus[c], Lv = Lvs[c];
-      const R wu = sm.u[c][0][e];
-      // the stage input the combination uses: first moments as modified by
-      // Step 1 (stored, the default), or unmodified (variant)
-      const R wvm = sm.vl[c][e - 1];
-      const R wv = (a.variant & HWENO_VARIANT_RAW_COMBINE) ? sm.u[c][1][e] : wvm;
-      R ou, ov;
-      if (a.stage == 0) {
-        ou = Lu;
-        ov = Lv;
-      } else {
-        const R rdt = dt;
-        const R su = wu + rdt * Lu, sv = wv + rdt * Lv;
-        if (a.stage == 1) {
-          ou = su;
-          ov = sv;
-        } else {
-          const R cb = a.stage == 2 ? R(0.25) : R(2.0 / 3.0);
-          ou = rk_combine(cb, u0c[c][0], su);
-          ov = rk_combine(cb, u0c[c][1], sv);
-        }
-      }
-      R* out = static_cast<R*>(a.out);
-      out[(2 * c + 0) * n + i] = ou;
-      out[(2 * c + 1) * n + i] = ov;
-      if (a.lim_out) {
-        R* lo = static_cast<R*>(a.lim_out);
-        lo[(2 * c + 0) * n + i] = wu;
-        lo[(2 * c + 1) * n + i] = a.stage == 0 ? wvm : wv;  // rhs mode: the modified moment
-      }
-      if (!isfinite(ou) || !isfinite(ov)) bad |= ST_NONFINITE;
-      Uo[c] = ou;
-    }
-    if (a.flags_out) a.flags_out[i] = (uint8_t)myflag;
-    if (a.stage > 0) {
-      speed = wave_speed<R, C>(gas, Uo);
-      if (!(speed == speed)) {
-        bad |= ST_NONPHYSICAL;
-        speed = R(0);
-      }
-    }
-  }
-  // 6. epilogue: the maximum wave speed of the output into the tile's slot
-  //    for the next alpha (a maximum does not depend on the order of the
-  //    atomics), the troubled count, the status bits.  Batches and grids of up
-  //    to kWarpAtomicTiles tiles fold each warp's values directly (no CTA
-  //    barrier on the latency-bound path); larger grids reduce over the CTA
-  //    first, so that the slots' atomic queues stay short.
-  R wmax = speed;
-  for (int o = 16; o > 0; o >>= 1) wmax = fmax(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
-  const int wcnt = __popc(__ballot_sync(0xffffffffu, myflag));
-  if (bad) atomicOr(&a.sc->status, bad);
-  double* const slot = static_cast<double*>(a.a_out) + (BATCH ? inst : tile % kAlphaSlots);
-  if (BATCH || a.ntile <= kWarpAtomicTiles) {
-    if (lane == 0) {
-      if (a.a_out) atomic_max_nonneg(slot, (double)wmax);
-      if (wcnt) atomicAdd(&a.sc->troubled, (unsigned long long)wcnt);
-    }
-    return;
-  }
-  if (lane == 0) {
-    sm.red[warp] = wmax;
-    sm.cnt[warp] = wcnt;
-  }
-  bar_sync(kBarCells, NT);
-  if (warp == 0) {
-    R m = lane < NW ? sm.red[lane] : R(0);
-    int c = lane < NW ? sm.cnt[lane] : 0;
-    for (int o = 16; o > 0; o >>= 1) {
-      m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-      c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
-    if (lane == 0) {
-      if (a.a_out) atomic_max_nonneg(slot, (double)m);
-      if (c) atomicAdd(&a.sc->troubled, (unsigned long long)c);
-    }
-  }
 }
 
 }  // namespace s1d

@@ -27,14 +27,14 @@ struct hweno_ctx {
   cudaStream_t cap = nullptr;        // private stream used only to capture graphs
   int C = 0, M = 0, n = 0, ntile = 0;  // n = cells; ntile = CTAs of one stage
   int dim = 1;
-  // 1D execution: threads per CTA of the stage kernels (a tile is nth1d - 6
-  // cells), and how hweno_step launches: per-stage launches in CUDA graphs
+  // 1D execution: threads per CTA of the stage kernels (stage1d_cells per tile),
+  // and how hweno_step launches: per-stage launches in CUDA graphs
   // (persist1d = 0), one persistent launch with a grid barrier per stage (1),
   // or one resident launch that keeps the tiles on chip (2, FP32 single
   // instance); hweno_autotune chooses
   int nth1d = 256, persist1d = 0;
   // the resident launch's geometry and cross-CTA buffers (allocated on first use)
-  int res_tile = 0, res_ncta = 0, res_cap = 0;
+  int res_nth = 0, res_tile = 0, res_ncta = 0, res_cap = 0;
   unsigned long long* res_halo = nullptr;     // tagged exchange words of the halos
   unsigned long long* res_entries = nullptr;  // and of the per-CTA maxima
   // small FP32 single instances: the cluster run's geometry (tile_cl = 0: not
@@ -54,7 +54,7 @@ struct hweno_ctx {
   int ntile_alpha = 0;               // CTAs of the wave-speed kernels (1D: kTile1D cells each; 2D: the stage tiles)
   unsigned* bar = nullptr;           // grid barrier of the persistent kernel
   std::vector<int> batch_nx;         // cells of each batch instance
-  std::vector<hw::BatchInst> batch_inst;
+  std::vector<hw::BatchTile> batch_inst;  // each instance's record (tile fields unset)
   double* tot_buf = nullptr;         // hweno_totals: partials, then the sums
   size_t elems = 0, esize = 0;
   void* U[3] = {nullptr, nullptr, nullptr};
@@ -70,9 +70,7 @@ struct hweno_ctx {
   std::string err;
   // batches of independent 1D instances
   int n_batch = 0;
-  int* d_tile_inst = nullptr;
-  int* d_tile_base = nullptr;
-  hw::BatchInst* d_binst = nullptr;
+  hw::BatchTile* d_btile = nullptr;
   hw::BatchScalars* d_bsc = nullptr;
   // adjoint: the tape of hweno_record and the scratch of hweno_backward
   struct Tape {
@@ -116,13 +114,28 @@ hweno_status fail(hweno_ctx* h, hweno_status st, const std::string& msg) {
       return fail((h), HWENO_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
+// CTAs of one 1D stage on n cells.
+int tiles1d(int n, int precision, int nth) {
+  const int T = hw::stage1d_cells(precision == HWENO_FP64, nth);
+  return (n + T - 1) / T;
+}
+
+// Threads per CTA of a single instance's FP32 stages, which run where the grid
+// is too large to be resident: 256 while two CTAs per SM hold it, then 128 (us
+// per stage with 128 / 256 / 512 threads: 100000 cells 5.9 / 5.1 / 5.7, 300000
+// 8.7 / 8.6 / 8.4, 1000000 23.5 / 27.3 / 30.9).
+int stage_threads(const hweno_ctx* h) {
+  if (h->esize == 8 || h->n_batch > 0) return h->nth1d;
+  return h->n <= 304 * hw::stage1d_cells(0, 256) ? 256 : 128;
+}
+
 hw::Stage1DArgs base_args(const hweno_ctx* h) {
   hw::Stage1DArgs a;
   memset(&a, 0, sizeof(a));
   const hweno_config& c = h->cfg;
   a.n = h->n;
-  a.ntile = h->ntile;
-  a.nth = h->nth1d;
+  a.nth = stage_threads(h);
+  a.ntile = a.nth == h->nth1d ? h->ntile : tiles1d(h->n, c.precision, a.nth);
   a.bc = c.bc;
   a.mode = c.troubled_mode;
   a.system = c.system;
@@ -136,9 +149,7 @@ hw::Stage1DArgs base_args(const hweno_ctx* h) {
   for (int k = 0; k < 3; ++k) a.gam[k] = c.lin_w[k];
   hw::finish_stage_args(a);
   if (h->n_batch > 0) {
-    a.tile_inst = h->d_tile_inst;
-    a.tile_base = h->d_tile_base;
-    a.binst = h->d_binst;
+    a.btile = h->d_btile;
     a.bsc = h->d_bsc;
   }
   return a;
@@ -294,15 +305,16 @@ cudaError_t enqueue_run1d(hweno_ctx* h, int nsteps, cudaStream_t s) {
   return hw::launch_run1d(r, s);
 }
 
-// Geometry of the resident launch for the handle's threads per CTA (res_tile =
-// 0 when it cannot run: FP64, batches, or too many cells to be co-resident),
-// and its buffers.
-cudaError_t prepare_resident(hweno_ctx* h) {
+// Geometry of the resident launch with nth threads per CTA (res_tile = 0 when it
+// cannot run: FP64, batches, or too many cells to be co-resident), and its
+// buffers.
+cudaError_t prepare_resident(hweno_ctx* h, int nth) {
   h->res_tile = h->res_ncta = 0;
+  h->res_nth = nth;
   if (h->dim != 1 || h->n_batch > 0 || h->cfg.precision == HWENO_FP64) return cudaSuccess;
-  if (h->nth1d != 256 && h->nth1d != 512) return cudaSuccess;
+  if (nth != 256 && nth != 512) return cudaSuccess;
   int tile = 0, ncta = 0;
-  cudaError_t e = hw::resident1d_geometry(h->cfg.system, h->nth1d, h->comp, h->n, &tile, &ncta);
+  cudaError_t e = hw::resident1d_geometry(h->cfg.system, nth, h->comp, h->n, &tile, &ncta);
   if (e != cudaSuccess || tile == 0) return e;
   if (ncta > h->res_cap) {
     if (h->res_halo) cudaFree(h->res_halo);
@@ -341,7 +353,7 @@ cudaError_t enqueue_resident1d(hweno_ctx* h, int nsteps, cudaStream_t s, int sil
   r.polls = polls;
   r.silent_cta = silent_cta;
   r.lo = h->comp ? h->Ulo : nullptr;
-  return hw::launch_resident1d(r, h->nth1d, h->res_ncta, s);
+  return hw::launch_resident1d(r, h->res_nth, h->res_ncta, s);
 }
 
 // nsteps Runge-Kutta steps of a small FP32 or float-pair handle in one launch
@@ -492,6 +504,20 @@ hweno_status check_scalars(hweno_ctx* h, hw::DevScalars* dev, hw::DevScalars* ho
   return HWENO_OK;
 }
 
+// The status of one hweno_rhs call.  Its scalars hold nothing but status bits that
+// matter (no time), so they are reset after a call that set one instead of
+// before every call.
+hweno_status check_rhs(hweno_ctx* h) {
+  hw::DevScalars s;
+  const hweno_status st = check_scalars(h, h->sc_rhs, &s);
+  if (st != HWENO_OK) {
+    const std::string err = h->err;
+    HW_CUDA(h, hw::launch_set_scalars(h->sc_rhs, 1, -1.0, h->stream));
+    h->err = err;
+  }
+  return st;
+}
+
 void free_ptr(void** p) {
   if (*p) cudaFree(*p);
   *p = nullptr;
@@ -567,30 +593,23 @@ hw::Adj2DArgs base_adj_args(const hweno_ctx* h) {
   return a;
 }
 
-// The tiles of every batch instance for stage CTAs of nth threads (nth - 6
-// cells per tile): tile -> instance and first cell, each instance's first
-// tile; replaces the previous tiling.
+// The tiles of every batch instance for stage CTAs of nth threads
+// (stage1d_cells per tile): tile -> instance and first cell, each instance's replaces
+// the previous tiling.
 cudaError_t batch_tiles(hweno_ctx* h, int nth) {
-  const int T = nth - 6;
-  std::vector<int> tinst, tbase;
-  for (int b = 0; b < h->n_batch; ++b) {
-    h->batch_inst[b].first_tile = (int)tinst.size();
+  const int T = hw::stage1d_cells(h->cfg.precision == HWENO_FP64, nth);
+  std::vector<hw::BatchTile> tiles;
+  for (int b = 0; b < h->n_batch; ++b)
     for (int base = 0; base < h->batch_nx[b]; base += T) {
-      tinst.push_back(b);
-      tbase.push_back(base);
+      tiles.push_back(h->batch_inst[b]);
+      tiles.back().base = base;
     }
-  }
-  if (h->d_tile_inst) cudaFree(h->d_tile_inst);
-  if (h->d_tile_base) cudaFree(h->d_tile_base);
-  h->d_tile_inst = h->d_tile_base = nullptr;
-  const size_t nt = tinst.size();
-  cudaError_t e = cudaMalloc(&h->d_tile_inst, sizeof(int) * nt);
-  if (e == cudaSuccess) e = cudaMalloc(&h->d_tile_base, sizeof(int) * nt);
-  if (e == cudaSuccess) e = cudaMemcpy(h->d_tile_inst, tinst.data(), sizeof(int) * nt, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(h->d_tile_base, tbase.data(), sizeof(int) * nt, cudaMemcpyHostToDevice);
+  if (h->d_btile) cudaFree(h->d_btile);
+  h->d_btile = nullptr;
+  const size_t nt = tiles.size();
+  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&h->d_btile), sizeof(hw::BatchTile) * nt);
   if (e == cudaSuccess)
-    e = cudaMemcpy(h->d_binst, h->batch_inst.data(), sizeof(hw::BatchInst) * h->n_batch,
-                   cudaMemcpyHostToDevice);
+    e = cudaMemcpy(h->d_btile, tiles.data(), sizeof(hw::BatchTile) * nt, cudaMemcpyHostToDevice);
   h->ntile = (int)nt;
   return e;
 }
@@ -651,7 +670,7 @@ hweno_status hweno_create(const hweno_config* cfg, void* cuda_stream, hweno_hand
     h->C = cfg->system == HWENO_EULER ? 3 : 1;
     h->M = 2;
     h->n = cfg->nx;
-    h->ntile = (h->n + h->nth1d - 7) / (h->nth1d - 6);
+    h->ntile = tiles1d(h->n, cfg->precision, h->nth1d);
     h->ntile_alpha = (h->n + hw::kTile1D - 1) / hw::kTile1D;
   }
   h->elems = (size_t)h->C * h->M * h->n;
@@ -674,6 +693,7 @@ hweno_status hweno_create(const hweno_config* cfg, void* cuda_stream, hweno_hand
   if (e == cudaSuccess) e = cudaMalloc(&h->sc_rhs, sizeof(hw::DevScalars));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = hw::launch_set_scalars(h->sc, 1, -1.0, h->stream);
+  if (e == cudaSuccess) e = hw::launch_set_scalars(h->sc_rhs, 1, -1.0, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) {
     std::string msg = std::string("allocation: ") + cudaGetErrorString(e);
@@ -690,7 +710,7 @@ hweno_status hweno_create(const hweno_config* cfg, void* cuda_stream, hweno_hand
   }
   if (h->comp && h->dim == 1) {  // the resident launch only
     h->persist1d = 2;
-    e = prepare_resident(h);
+    e = prepare_resident(h, h->nth1d);
     if (e != cudaSuccess || h->res_tile == 0) {
       std::string msg = e != cudaSuccess ? std::string("resident launch: ") + cudaGetErrorString(e)
                                          : std::string("HWENO_FP32C runs as the resident launch, "
@@ -779,10 +799,24 @@ hweno_status hweno_step(hweno_handle h, int nsteps, double t_final, double* t_ou
       HW_CUDA(h, e);
     }
   }
-  if (h->dim == 1 && h->persist1d == 2) {
-    if (left > 0) HW_CUDA(h, enqueue_resident1d(h, left, h->stream));
-    left = 0;
-  } else if (h->dim == 1 && h->persist1d) {
+  if (h->dim == 1 && h->n_batch == 0 && h->esize == 4 && left > 0) {
+    // FP32: the resident launch where the grid fits, also when the handle is set
+    // to another launch (5000 to 65536 cells: 2.9-3.1 us per stage against
+    // 3.4-3.9 by graphs of a cell per thread, 4.3-4.6 of two, 4.0-4.2 persistent)
+    const int nth = h->persist1d == 2 ? h->nth1d : 256;
+    if (h->res_nth != nth) HW_CUDA(h, prepare_resident(h, nth));
+    if (h->res_tile > 0) {
+      cudaError_t e = enqueue_resident1d(h, left, h->stream);
+      if (e == cudaErrorCooperativeLaunchTooLarge && h->persist1d != 2) {
+        cudaGetLastError();
+        h->res_tile = 0;
+      } else {
+        HW_CUDA(h, e);
+        left = 0;
+      }
+    }
+  }
+  if (h->dim == 1 && h->persist1d == 1 && h->esize == 8) {  // (FP32: by stages, below)
     if (left > 0) HW_CUDA(h, enqueue_run1d(h, left, h->stream));
     left = 0;
   }
@@ -815,7 +849,6 @@ hweno_status hweno_rhs(hweno_handle h, const void* in, void* out, uint8_t* flags
   if (!in || !out) return fail(h, HWENO_ERR_ARG, "in and out must be device pointers");
   if (in == out || (ulim_out && (ulim_out == in || ulim_out == out)))
     return fail(h, HWENO_ERR_ARG, "in, out and ulim_out must not overlap");
-  HW_CUDA(h, hw::launch_set_scalars(h->sc_rhs, 1, -1.0, h->stream));
   if (h->dim == 2) {
     HW_CUDA(h, hw::launch_alpha2d(in, h->part_rhs, h->cfg.nx, h->cfg.ny, h->cfg.system,
                                   h->cfg.precision == HWENO_FP64, h->cfg.gas_gamma, h->sc_rhs, 0,
@@ -830,8 +863,7 @@ hweno_status hweno_rhs(hweno_handle h, const void* in, void* out, uint8_t* flags
     a.sc = h->sc_rhs;
     a.flags_out = flags_out;
     HW_CUDA(h, hw::launch_stage2d(a, h->stream));
-    hw::DevScalars s2;
-    return check_scalars(h, h->sc_rhs, &s2);
+    return check_rhs(h);
   }
   HW_CUDA(h, hw::launch_alpha1d(in, h->part_rhs, h->n, h->ntile_alpha, h->cfg.system,
                                 h->cfg.precision == HWENO_FP64, h->cfg.gas_gamma, h->sc_rhs, 0,
@@ -848,8 +880,7 @@ hweno_status hweno_rhs(hweno_handle h, const void* in, void* out, uint8_t* flags
   a.flags_out = flags_out;
   hw::rhs_tiles1d(a);
   HW_CUDA(h, hw::launch_stage1d(a, h->stream));
-  hw::DevScalars s;
-  return check_scalars(h, h->sc_rhs, &s);
+  return check_rhs(h);
 }
 
 hweno_status hweno_get_state(hweno_handle h, void* out, int dtype, int on_device) {
@@ -922,9 +953,7 @@ void hweno_destroy(hweno_handle h) {
   for (int k = 0; k < 2; ++k)
     if (h->Ulo_s[k]) cudaFree(h->Ulo_s[k]);
   if (h->tot_buf) cudaFree(h->tot_buf);
-  if (h->d_tile_inst) cudaFree(h->d_tile_inst);
-  if (h->d_tile_base) cudaFree(h->d_tile_base);
-  if (h->d_binst) cudaFree(h->d_binst);
+  if (h->d_btile) cudaFree(h->d_btile);
   if (h->d_bsc) cudaFree(h->d_bsc);
   free_tape(h, true);
   if (h->cap) cudaStreamDestroy(h->cap);
@@ -961,22 +990,21 @@ hweno_status hweno_create_batch(const hweno_config* cfg, int n_batch, const int*
   h->batch_nx.assign(nx, nx + n_batch);
   h->batch_inst.resize(n_batch);
   for (int b = 0; b < n_batch; ++b) {
-    hw::BatchInst& bi = h->batch_inst[b];
+    hw::BatchTile& bi = h->batch_inst[b];
     const double dx = (c.x1 - c.x0) / nx[b];
     bi.off = (long long)C * 2 * cells;
     bi.n = nx[b];
-    bi.first_tile = 0;
+    bi.base = 0;
+    bi.inst = b;
     bi.inv_dx = 1.0 / dx;
     bi.h = 0.5 * dx;
     bi.cfl_dx = c.cfl * dx;
     bi.inv_dx_f = (float)bi.inv_dx;
     bi.hthr_f = (float)(c.kxrcf_threshold * bi.h);
-    bi.cfl_dx_f = (float)bi.cfl_dx;
     bi.hthr_lo_f = (float)(c.kxrcf_threshold * bi.h - (double)bi.hthr_f);
     cells += nx[b];
   }
-  cudaError_t e = cudaMalloc(&h->d_binst, sizeof(hw::BatchInst) * n_batch);
-  if (e == cudaSuccess) e = cudaMalloc(&h->d_bsc, sizeof(hw::BatchScalars) * n_batch);
+  cudaError_t e = cudaMalloc(&h->d_bsc, sizeof(hw::BatchScalars) * n_batch);
   if (e == cudaSuccess) e = batch_tiles(h, h->nth1d);
   // one alpha slot per instance in each of the three rotating buffers
   for (int r = 0; r < 3 && e == cudaSuccess && n_batch > 2 * hw::kAlphaSlots; ++r) {
@@ -1234,10 +1262,10 @@ hweno_status hweno_set_execution(hweno_handle h, int threads, int persistent) {
   if (h->n_batch > 0) {
     HW_CUDA(h, batch_tiles(h, threads));
   } else {
-    h->ntile = (h->n + threads - 7) / (threads - 6);
+    h->ntile = tiles1d(h->n, h->cfg.precision, threads);
   }
   if (persistent == 2) {
-    HW_CUDA(h, prepare_resident(h));
+    HW_CUDA(h, prepare_resident(h, threads));
     if (h->res_tile == 0) {
       h->persist1d = 0;
       return fail(h, HWENO_ERR_ARG,
@@ -1292,8 +1320,8 @@ hweno_status hweno_autotune(hweno_handle h, int nsteps_trial, int* choice_out) {
     h->nth1d = nth;
     h->persist1d = persist;
     if (h->n_batch > 0) return batch_tiles(h, nth);
-    h->ntile = (h->n + nth - 7) / (nth - 6);
-    if (persist == 2) return prepare_resident(h);
+    h->ntile = tiles1d(h->n, h->cfg.precision, nth);
+    if (persist == 2) return prepare_resident(h, nth);
     return cudaSuccess;
   };
   cudaError_t e = copy_all(true);
@@ -1394,6 +1422,7 @@ hweno_status hweno_check_resident(hweno_handle h, int nsteps, int silent_cta, un
   if (nsteps < 1 || silent_cta < -1 || silent_cta >= h->res_ncta || polls < 1u)
     return fail(h, HWENO_ERR_ARG,
                 "hweno_check_resident: need nsteps >= 1, -1 <= silent_cta < CTAs, polls >= 1");
+  if (h->res_nth != h->nth1d) HW_CUDA(h, prepare_resident(h, h->nth1d));
   HW_CUDA(h, hw::launch_set_scalars(h->sc, 0, -1.0, h->stream));
   HW_CUDA(h, enqueue_resident1d(h, nsteps, h->stream, silent_cta, polls));
   hw::DevScalars host;

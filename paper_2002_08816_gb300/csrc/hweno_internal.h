@@ -11,13 +11,15 @@
 
 namespace hw {
 
-// One instance of a batch of independent 1D problems.
-struct BatchInst {
+// One tile of a batch of independent 1D problems: its instance, first cell, and
+// the instance's geometry (all in one record, so that a CTA that finds its tile
+// needs one round trip to memory before its first load of data).
+struct BatchTile {
   long long off;           // element offset of the instance's state in the batch buffer
-  int n;                   // cells
-  int first_tile;          // first tile of the instance
+  int n, base, inst;       // cells of the instance, first cell of the tile, the instance
+  float inv_dx_f;
   double inv_dx, h, cfl_dx;
-  float inv_dx_f, hthr_f, cfl_dx_f, hthr_lo_f;
+  float hthr_f, hthr_lo_f;
 };
 
 // Time bookkeeping of one instance.
@@ -44,8 +46,8 @@ struct Stage1DArgs {
   uint8_t* flags_out;    // troubled flags of the own cells (nullable)
   int n;                 // cells
   int ntile;             // tiles (= CTAs of a per-stage launch)
-  int nth;               // threads per CTA of the stage kernels: 128, 256 (also 0) or 512;
-                         // a tile is nth - 6 cells (FP64, no batch: also 32, a 26-cell tile)
+  int nth;               // threads per CTA of the stage kernels: 128, 256 (also 0) or 512
+                         // (stage1d_cells); FP64, no batch: also 32, a 26-cell tile
   int stage;             // 1, 2, 3; 0 = rhs mode
   int bc;                // 0 periodic, 1 outflow
   int mode;              // 0 hybrid, 1 all, 2 none
@@ -62,10 +64,7 @@ struct Stage1DArgs {
   float hthr;            // (float)(thr * h)
   float hthr_lo;         // (float)(thr * h - hthr): thr * h = hthr + hthr_lo to ~2^-48
   float f32[7];          // FP32 copies: gamma_0..2, eps, gas_gamma, 1/dx, cfl*dx
-  // batches of independent instances (nullable): tile -> instance, first cell
-  const int* tile_inst;
-  const int* tile_base;
-  const BatchInst* binst;
+  const BatchTile* btile;  // batches of independent instances (nullable)
   BatchScalars* bsc;
 };
 
@@ -86,8 +85,14 @@ inline void finish_stage_args(Stage1DArgs& a) {
 }
 
 constexpr int kAlphaSlots = 64;  // slots that carry alpha between stages
-constexpr int kTile1D = 250;     // cells per CTA of the 1D kernels
-constexpr int kThreads1D = 256;  // threads per CTA (tile + 3-cell halo per side)
+constexpr int kTile1D = 250;     // cells per CTA of the 1D wave-speed kernels
+constexpr int kThreads1D = 256;  // their threads per CTA
+// Cells per tile of the 1D stage kernels with nth cell threads: FP64 nth less the
+// halo, FP32 two such halves (two cells per thread); 0 threads: 256.
+inline int stage1d_cells(int fp64, int nth) {
+  const int w = (nth ? nth : 256) - 6;
+  return fp64 ? w : 2 * w;
+}
 
 // KXRCF constants of the 2D reading, derived on the host
 struct Kx2 {
@@ -273,7 +278,7 @@ cudaError_t launch_run1d(const Run1DArgs& r, cudaStream_t s);
 // hweno_check_barrier's launch; *too_many when ctas cannot all be resident
 cudaError_t launch_barrier_check(int ctas, int meetings, int missing, unsigned polls,
                                  unsigned* bar, DevScalars* sc, cudaStream_t s, bool* too_many);
-// Batched variants: one launch over all instances (a.tile_inst != nullptr);
+// Batched variants: one launch over all instances (a.btile != nullptr);
 // alpha slots are one per instance.
 cudaError_t launch_alpha1d_batch(const Stage1DArgs& a, cudaStream_t s);
 cudaError_t launch_batch_scalars(BatchScalars* bsc, int n_inst, int reset, double t_final,

@@ -99,7 +99,8 @@ hweno_status hweno_rhs1d_noalloc(const hweno_config* cfg, void* cuda_stream, con
     a.sc = sc;
     a.flags_out = flags_out;
     a.n = n;
-    a.ntile = ntile;
+    const int cells = hw::stage1d_cells(fp64, 0);
+    a.ntile = (n + cells - 1) / cells;
     a.stage = 0;
     a.bc = cfg->bc;
     a.mode = cfg->troubled_mode;
