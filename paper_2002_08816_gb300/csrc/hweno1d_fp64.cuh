@@ -50,34 +50,6 @@ struct Smem64 {
   int ntb, nhw;
 };
 
-__device__ __forceinline__ int hi_of(double x) { return __double2hiint(x); }
-__device__ __forceinline__ bool finite_bits(double x) { return (hi_of(x) & 0x7ff00000) != 0x7ff00000; }
-// x >= 0 and x > 0 without an FP64 instruction (NaN: false; -0 >= 0)
-__device__ __forceinline__ bool ge0(double x) {
-  const long long b = __double_as_longlong(x);
-  return b >= 0 ? b <= 0x7ff0000000000000ll : (b << 1) == 0;
-}
-__device__ __forceinline__ bool gt0(double x) {
-  const long long b = __double_as_longlong(x);
-  return b > 0 && b <= 0x7ff0000000000000ll;
-}
-__device__ __forceinline__ bool inflow_left(double rho, double m) {
-  return gt0(rho) ? ge0(m) : (m / rho >= 0.0);
-}
-
-// x truncated to FP32 by its bits (relative error < 2^-23); 0 below 2^-100,
-// NaN from 2^100 on (and for infinities and NaN): a comparison then decides
-// nothing and the FP64 form is taken.
-__device__ __forceinline__ float trunc32(double x) {
-  const int hi = __double2hiint(x), lo = __double2loint(x);
-  const int ex = (hi >> 20) & 0x7ff;
-  unsigned b = ((unsigned)hi & 0x80000000u) | (((unsigned)(hi & 0x7fffffff) - 0x38000000u) << 3) |
-               ((unsigned)lo >> 29);
-  if (ex < 923) b = 0u;
-  if (ex >= 1123) b = 0x7fc00000u;
-  return __uint_as_float(b);
-}
-
 // kxrcf_troubled(double ...) with the FP32 test in front: the truncated terms
 // carry 2^-23 S, the FP32 jump four roundings (together below 8e-7 S, S as
 // in the FP32 form), the threshold three roundings and a truncation (7e-7).

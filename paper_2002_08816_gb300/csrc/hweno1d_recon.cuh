@@ -301,4 +301,9 @@ __device__ __forceinline__ bool inflow_left(R rho, R m) {
   return rho > R(0) ? (m >= R(0)) : (m / rho >= R(0));
 }
 
+// FP64 data: the same without an FP64 instruction.
+__device__ __forceinline__ bool inflow_left(double rho, double m) {
+  return gt0(rho) ? ge0(m) : (m / rho >= 0.0);
+}
+
 }  // namespace hw

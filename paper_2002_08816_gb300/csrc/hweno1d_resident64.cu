@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(NTH + 32, 2) resident64_kernel(Resident1DArgs 
       }
       un[c][0][e] = ou;
       un[c][1][e] = ov;
-      if (!f64::finite_bits(ou) || !f64::finite_bits(ov)) bad |= ST_NONFINITE;
+      if (!is_finite(ou) || !is_finite(ov)) bad |= ST_NONFINITE;
       const int ps = i < 3 ? i : (i >= Tq - 3 ? 3 + i - (Tq - 3) : -1);
       if (ps >= 0) {  // the neighbours' halo
         u64* dst = hal + ((size_t)q * 2 + (s & 1)) * HS + ps * (C * NV) + c * NV;

@@ -87,7 +87,7 @@ __device__ __forceinline__ void stage64_tile(Stage1DArgs a, const int tile, Smem
       lim[gu] = wu;
       lim[gv] = a.stage == 0 ? wvm : wv;  // rhs mode: the modified moment
     }
-    if (!finite_bits(ou) || !finite_bits(ov)) bad |= ST_NONFINITE;
+    if (!is_finite(ou) || !is_finite(ov)) bad |= ST_NONFINITE;
     if (c == 0 && a.flags_out) a.flags_out[base + i] = sm.fl[e];
   }
   if (a.stage > 0) {

@@ -33,6 +33,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include "hweno1d_fields.cuh"
 #include "hweno1d_recon.cuh"
 #include "hweno2d_common.cuh"
 #include "hweno_device.cuh"
@@ -42,20 +43,21 @@
 namespace hw {
 namespace {
 
-constexpr int TX = 32, TY = 8;  // cells per CTA of the stage and wave-speed kernels (a warp per row)
-constexpr int NT = kThreads2D;
-constexpr int NW = NT / 32;
+// Cells per CTA: 32 in x (a warp per row), TY rows of the stage kernel (8 or 4,
+// stage2d_rows), TYW of the wave-speed kernels.
+constexpr int TX = 32, TYW = 8;
+constexpr int NTW = TX * TYW, NWW = NTW / 32;
 // raw tile: a 3-cell halo, and in x one more column on the left so that the
 // tile's first column bx0 - 4 is 16-byte aligned (TMA); own-tile cell (ci, cj)
 // is raw (ci + OXR, cj + OYR)
-constexpr int RX = TX + 8, RY = TY + 6;
+constexpr int RX = TX + 8;
 constexpr int OXR = 4, OYR = 3;
-constexpr int LX = TX + 4, LY = TY + 4;  // flags and modified moments, 2-cell halo
+constexpr int LX = TX + 4;                // flags and modified moments, 2-cell halo
 constexpr unsigned kTmaPolls = 1u << 20;  // mbarrier polls before a tile copy is given up
-static_assert(TX * TY == NT, "one own cell per thread");
 
-template <typename R, int C, int NG, bool COMP = false>
+template <typename R, int C, int NG, bool COMP, int TY>
 struct Smem2D {
+  static constexpr int NW = TX * TY / 32, RY = TY + 6, LY = TY + 4;
   static constexpr int kPadX = 1;  // raw index of flag-grid column lx: lx + 2
   // the limiter's results go to `lim` by work-list slot (and are written into
   // u once every cell's flag and limiter has read the raw moments)
@@ -65,8 +67,10 @@ struct Smem2D {
   alignas(128) R u[C][3][RY][RX];
   // HWENO_FP32C: the low parts of the stage input's averages (a second box)
   alignas(128) R ulo[COMP ? C : 1][COMP ? RY : 1][COMP ? RX : 1];
-  R lim[C == 4 ? LX * LY : 1][C][2];  // Euler: modified x-, y-moments by list slot
-  R xf[C][2 * NG][TY][TX + 2];  // x-face values (left NG, right NG) of cells -1..TX
+  union {
+    R xf[C][2 * NG][TY][TX + 2];  // x-face values (left NG, right NG) of cells -1..TX
+    R lim[C == 4 ? LX * LY : 1][C][2];  // Step 4, Euler: modified x-, y-moments by list slot
+  };
   R yf[C][2 * NG][TY + 2][TX];  // y-face values (bottom NG, top NG) of cells -1..TY
   uint8_t fl[LY][LX];
   R red[2][NW];
@@ -138,6 +142,22 @@ __device__ __forceinline__ bool kxrcf2_troubled(float u0, float v0, float w0, fl
 __device__ __forceinline__ bool kxrcf2_troubled(double u0, double v0, double w0, double uxn,
                                                 double vxn, double uyn, double wyn, bool lowx,
                                                 bool lowy, const Kx2& k) {
+  {
+    // decided in FP32 on the truncated data where the error bound allows (no FP64
+    // instruction): as the FP32 form above, with the truncations' 2^-23 added
+    const float fu = trunc32(u0), fv = trunc32(v0), fw = trunc32(w0);
+    const float gx = trunc32(uxn), gvx = trunc32(vxn), gy = trunc32(uyn), gwy = trunc32(wyn);
+    const float sx6 = lowx ? -6.0f : 6.0f, sy6 = lowy ? -6.0f : 6.0f;
+    const float jxf = fmaf(sx6, fv, fu) - fmaf(-sx6, gvx, gx);
+    const float jyf = fmaf(sy6, fw, fu) - fmaf(-sy6, gwy, gy);
+    const float sx = fabsf(fu) + 6.0f * fabsf(fv) + fabsf(gx) + 6.0f * fabsf(gvx);
+    const float sy = fabsf(fu) + 6.0f * fabsf(fw) + fabsf(gy) + 6.0f * fabsf(gwy);
+    const float numf = fabsf(k.fdy * jxf + k.fdx * jyf);
+    const float e = 1.3e-6f * (k.fdy * sx + k.fdx * sy) + 1e-28f;
+    const float r = k.fthr_den * fmaxf(fabsf(fu), 1e-12f);
+    if (numf - e > r * (1.0f + 8.0e-7f)) return true;   // (NaN decides nothing)
+    if (numf + e < r * (1.0f - 8.0e-7f)) return false;
+  }
   const double jx = jump64(u0, v0, uxn, vxn, lowx);
   const double jy = jump64(u0, w0, uyn, wyn, lowy);
   const double num = __dadd_rn(__dmul_rn(k.dy, jx), __dmul_rn(k.dx, jy));
@@ -367,13 +387,125 @@ __device__ __noinline__ void hweno_faces_euler2d(S& sm, int ci, int cj, int p_lo
   }
 }
 
-template <typename R, int C, int NG, bool COMP>
-__global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
+// hweno_faces_euler2d in FP64 for the n listed items: (item, field) on four
+// consecutive lanes, the two directions on different warps.  An FP64 warp
+// instruction takes a sub-partition 64 cycles however few lanes work, and an
+// item is one long chain (2 directions x 4 fields), so a tile's few items as
+// one thread each left a single warp with ~6000 such instructions while the
+// rest of the SM waited; a task has ~550.
+template <int NG, int NT, typename S, typename F>
+__device__ __noinline__ void hweno_tasks_euler2d(S& sm, int n, F item_of, double g0, double g1, double g2,
+                                                 double g3, double g4, double eps, double gas,
+                                                 bool mean_eigen) {
+  const double gam[5] = {g0, g1, g2, g3, g4};
+  const int lane = threadIdx.x & 31, f = lane & 3, base = lane & ~3;
+  const int dir = (threadIdx.x >> 5) & 1;
+  for (int q0 = (threadIdx.x >> 6) * 8; q0 < n; q0 += NT / 64 * 8) {  // uniform over the warp
+    const int q = q0 + (lane >> 2);
+    int ci, cj, p_lo, p_hi;
+    item_of(sm.hwl[q < n ? q : q0], ci, cj, p_lo, p_hi);
+    for (int side = 0; side < (mean_eigen ? 2 : 1); ++side) {
+      const int lo = dir * 2 * NG + side * NG, hi = lo + (mean_eigen ? NG : 2 * NG);
+      const int plo = max(p_lo, lo), phi = q < n ? min(p_hi, hi) : plo;
+      if (!__any_sync(0xffffffffu, plo < phi)) continue;
+      double U[4];
+      const int dx = mean_eigen && dir == 0 ? 2 * side - 1 : 0, dy = mean_eigen && dir == 1 ? 2 * side - 1 : 0;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        U[c] = sm.u[c][0][cj + OYR][ci + OXR];
+        if (mean_eigen) U[c] = 0.5 * (U[c] + sm.u[c][0][cj + OYR + dy][ci + OXR + dx]);
+      }
+      double Rm[4][4], Lm[4][4], l[4], r[4];
+      Euler2D<double>::eigen(gas, U, dir, Rm, Lm);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {  // the row of field f; for component f, its row of Rm
+        l[c] = f == 0 ? Lm[0][c] : f == 1 ? Lm[1][c] : f == 2 ? Lm[2][c] : Lm[3][c];
+        r[c] = f == 0 ? Rm[0][c] : f == 1 ? Rm[1][c] : f == 2 ? Rm[2][c] : Rm[3][c];
+      }
+      double e[19], ch[2 * NG];
+#pragma unroll
+      for (int k = 0; k < 19; ++k) e[k] = 0.0;
+#pragma unroll 1
+      for (int c = 0; c < 4; ++c) {
+        double t[19];
+        const double lc = c == 0 ? l[0] : c == 1 ? l[1] : c == 2 ? l[2] : l[3];
+        gather19(sm, c, ci, cj, t);
+#pragma unroll
+        for (int k = 0; k < 19; ++k) e[k] = fma(lc, t[k], e[k]);
+      }
+      if (dir == 0) hweno2d_dir_faces<NG, 0>(e, gam, eps, ch);
+      else hweno2d_dir_faces<NG, 1>(e, gam, eps, ch);
+      // component f at the points: sum over the fields, which the item's lanes hold
+#pragma unroll
+      for (int p = 0; p < 2 * NG; ++p) {
+        double v = 0.0;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) v = fma(r[g], __shfl_sync(0xffffffffu, ch[p], base + g), v);
+        const int pt = dir * 2 * NG + p;
+        if (pt >= plo && pt < phi) {
+          if (dir == 0) store_point(sm, f, p, ci, cj, v);
+          else store_point(sm, f, 2 * NG + p, ci, cj, v);
+        }
+      }
+    }
+  }
+}
+
+// limit_euler2d in FP64 for the listed troubled cells, the same way.
+template <int NT, int LX_, typename S>
+__device__ __noinline__ void limit_tasks_euler2d(S& sm, int n, double g0, double g1, double g2, double eps,
+                                                 double gas) {
+  const double gam[3] = {g0, g1, g2};
+  const int lane = threadIdx.x & 31, f = lane & 3, dir = (lane >> 2) & 1, base = lane & ~3;
+  for (int q0 = (threadIdx.x >> 5) * 4; q0 < n; q0 += NT / 32 * 4) {
+    const int q = q0 + (lane >> 3);
+    const int k = sm.tbl[q < n ? q : q0];
+    const int rx = k % LX_ + 1 + S::kPadX, ry = k / LX_ + 1;
+    const int sx = dir == 0 ? 1 : 0, sy = 1 - sx, mom = 1 + dir;
+    double U[4], Rm[4][4], Lm[4][4], l[4], r[4], w[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) U[c] = sm.u[c][0][ry][rx];
+    Euler2D<double>::eigen(gas, U, dir, Rm, Lm);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      l[c] = f == 0 ? Lm[0][c] : f == 1 ? Lm[1][c] : f == 2 ? Lm[2][c] : Lm[3][c];
+      r[c] = f == 0 ? Rm[0][c] : f == 1 ? Rm[1][c] : f == 2 ? Rm[2][c] : Rm[3][c];
+      w[0] = fma(l[c], sm.u[c][0][ry - sy][rx - sx], w[0]);
+      w[1] = fma(l[c], U[c], w[1]);
+      w[2] = fma(l[c], sm.u[c][0][ry + sy][rx + sx], w[2]);
+      w[3] = fma(l[c], sm.u[c][mom][ry - sy][rx - sx], w[3]);
+      w[4] = fma(l[c], sm.u[c][mom][ry + sy][rx + sx], w[4]);
+    }
+    const double m = fld::limit_moment(w[0], w[1], w[2], w[3], w[4], gam, eps);
+    double v = 0.0;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) v = fma(r[g], __shfl_sync(0xffffffffu, m, base + g), v);
+    if (q < n) sm.lim[q][f][dir] = v;
+  }
+}
+
+// CTAs per SM the kernel is built for.  FP32 at 128 registers holds two; where its
+// shared memory leaves room for more (Euler with 2 Gauss points: three, Burgers:
+// four), a build at 80 or 64 registers with those is the faster one on grids of
+// several waves of tiles (DENSE; 4096 x 4096 Euler, 2 points 18.7 -> 14.6 ms for 4
+// steps; 2048 x 2048 Burgers, 3 points 2.50 -> 1.63), and the slower one on a
+// single wave, which is bound by a tile's own chain (240 x 240 Euler, 2 points,
+// 30 steps 1.08 -> 1.15): stage2d_dense decides.
+template <typename R, int C, int NG, bool DENSE, int TY>
+constexpr int stage2d_ctas() {
+  return (sizeof(R) == 8 ? 1 : !DENSE ? 2 : C == 1 ? 4 : 3) * 8 / TY;
+}
+template <typename R, int C, int NG>
+constexpr bool has_dense() { return sizeof(R) == 4 && (C == 1 || NG == 2); }
+
+template <typename R, int C, int NG, bool COMP, bool DENSE, int TY>
+__global__ void __launch_bounds__(TX * TY, (stage2d_ctas<R, C, NG, DENSE, TY>()))
     stage2d_kernel(Stage2DArgs a, const __grid_constant__ CUtensorMap tile_map,
                    const __grid_constant__ CUtensorMap lo_map) {
   static_assert(!COMP || sizeof(R) == 4, "the float-pair averages are FP32");
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  using SM = Smem2D<R, C, NG, COMP>;
+  using SM = Smem2D<R, C, NG, COMP, TY>;
+  constexpr int NT = TX * TY, NW = SM::NW, RY = SM::RY, LY = SM::LY;  // one own cell per thread
   SM& sm = *reinterpret_cast<SM*>(smem_raw);
   constexpr int NF = 4 * NG, NI = NG * NG;
   // FP32 Euler: the linear p0 maps take two components at once (packed FP32)
@@ -499,9 +631,11 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
   // ---- 2. Step 4 on the tile plus 2 halo cells; the modified first moments
   // of the troubled cells replace the raw ones in the tile only after every
   // flag and limiter has read the raw ones
-  static_assert(LX * LY <= 2 * NT, "two cells of Step 4 per thread at most");
-  R hv[2][2];       // Burgers: the modified moments of this thread's troubled cells
-  int hk[2] = {-1, -1};
+  constexpr int kRounds = (LX * LY + NT - 1) / NT;  // cells of Step 4 per thread at most
+  R hv[kRounds][2];  // Burgers: the modified moments of this thread's troubled cells
+  int hk[kRounds];
+#pragma unroll
+  for (int j = 0; j < kRounds; ++j) hk[j] = -1;
   int it = 0;
   for (int k = tid; k < LX * LY; k += NT, ++it) {
     const int lx = k % LX, ly = k / LX;
@@ -567,10 +701,13 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
   // no interface item of the tile needs HWENO and none tests its stencil
   bool tile_troubled;
   if constexpr (C == 1) {
-    tile_troubled = __syncthreads_or(hk[0] >= 0 || hk[1] >= 0);
+    bool mine = false;
+#pragma unroll
+    for (int j = 0; j < kRounds; ++j) mine |= hk[j] >= 0;
+    tile_troubled = __syncthreads_or(mine);
     if (tile_troubled) {
 #pragma unroll
-      for (int j = 0; j < 2; ++j)
+      for (int j = 0; j < kRounds; ++j)
         if (hk[j] >= 0) {
           const int rx = hk[j] % LX + 1 + SM::kPadX, ry = hk[j] / LX + 1;
           sm.u[0][1][ry][rx] = hv[j][0];
@@ -582,7 +719,8 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
     __syncthreads();
     tile_troubled = sm.ntb > 0;
     if (tile_troubled) {
-      for (int q = tid; q < sm.ntb; q += NT) {
+      if constexpr (sizeof(R) == 8) limit_tasks_euler2d<NT, LX>(sm, sm.ntb, gam[0], gam[1], gam[2], eps, gas);
+      else for (int q = tid; q < sm.ntb; q += NT) {
         const int k = sm.tbl[q];
         limit_euler2d(sm, k % LX, k / LX, q, gam[0], gam[1], gam[2], gam[3], gam[4], eps, gas);
       }
@@ -603,9 +741,12 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
   // ---- 3. interface values of the own cells (all faces) and of the cross
   //         halo (left column: right face, right column: left face, bottom
   //         row: top face, top row: bottom face)
-  //         by linear p0; the items whose stencil holds a troubled cell are
-  //         listed and reconstructed by HWENO on consecutive threads below
-  //         (the same arithmetic, fewer warps diverging on it)
+  //         by linear p0, and of the own cells the interior points (Step 5.3)
+  //         with their volume integrals, from the same parity classes (the
+  //         second gather and fold of phase 4 cost more than the 2 C sums held
+  //         through the barrier); the items whose stencil holds a troubled
+  //         cell are listed and reconstructed by HWENO on consecutive threads
+  //         below (the same arithmetic, fewer warps diverging on it)
   auto item_of = [](int item, int& ci, int& cj, int& p_lo, int& p_hi) {
     if (item < TX * TY) {  // own cell: every interface point
       ci = item % TX; cj = item / TX; p_lo = 0; p_hi = NF;
@@ -617,45 +758,139 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
       else { ci = TX; cj = h - 2 * TX - TY; p_lo = 0; p_hi = NG; }
     }
   };
-  for (int item = tid; item < TX * TY + 2 * TX + 2 * TY; item += NT) {
-    int ci, cj, p_lo, p_hi;  // own-tile coordinates of the cell, point range
-    item_of(item, ci, cj, p_lo, p_hi);
+  constexpr double r15 = 0.38729833462074168852;  // sqrt(15)/10
+  constexpr double r3 = 0.28867513459481288225;   // sqrt(3)/6
+  const R gw[3] = {NG == 3 ? R(5.0 / 18.0) : R(0.5), NG == 3 ? R(4.0 / 9.0) : R(0.5), R(5.0 / 18.0)};
+  const R gx[3] = {NG == 3 ? R(-r15) : R(-r3), NG == 3 ? R(0) : R(r3), R(r15)};
+  const int ci = ox, cj = oy;  // the own cell, as the item of this thread
+  // COMP: every point value is an increment over the own cell's hi B, every
+  // flux an increment over f(B) (the base cancels from Eq. (ode2) exactly)
+  R B[C];
+#pragma unroll
+  for (int c = 0; c < C; ++c) B[c] = sm.u[c][0][cj + OYR][ci + OXR];
+  auto flux = [&](const R* U, int dir, R* F) {
+    if constexpr (COMP) flux_inc2<C>(gas, B, U, dir, F);
+    else phys_flux2<R, C>(gas, U, dir, F);
+  };
+  R Fv[C], Gv[C];  // the volume integrals of Eq. (ode2)
+#pragma unroll
+  for (int c = 0; c < C; ++c) Fv[c] = Gv[c] = R(0);
+  using T = typename PairOf<R, kPacked>::type;
+  auto near_troubled = [&](int i, int j) {
     bool hw = false;
     if (tile_troubled) {
 #pragma unroll
       for (int dj = -1; dj <= 1; ++dj)
 #pragma unroll
-        for (int di = -1; di <= 1; ++di) hw |= sm.fl[cj + 2 + dj][ci + 2 + di] != 0;
+        for (int di = -1; di <= 1; ++di) hw |= sm.fl[j + 2 + dj][i + 2 + di] != 0;
     }
+    return hw;
+  };
+  // the values at the points [p_lo, p_hi) of component c (packed: c and c + 1)
+  // of cell (i, j) from its parity classes
+  auto faces = [&](const T* s, int c, int i, int j, int p_lo, int p_hi) {
+    if (p_lo < 2 * NG) {
+      T v[2 * NG];
+      p0s_xfaces<NG>(s, v);
+#pragma unroll
+      for (int p = 0; p < 2 * NG; ++p)
+        if (p >= p_lo && p < p_hi) store_points(sm, c, p, i, j, v[p]);
+    }
+    if (p_hi > 2 * NG) {
+      T v[2 * NG];
+      p0s_yfaces<NG>(s, v);
+#pragma unroll
+      for (int p = 0; p < 2 * NG; ++p)
+        if (p + 2 * NG >= p_lo && p + 2 * NG < p_hi) store_points(sm, c, p + 2 * NG, i, j, v[p]);
+    }
+  };
+  {
+    const bool hw = near_troubled(ci, cj);
+    R inter[C][NI];
+#pragma unroll
+    for (int c = 0; c < C; c += kPacked ? 2 : 1) {
+      T s[19], v[NI];
+      classes_of<COMP, kPacked>(sm, c, ci, cj, s);
+      if (!hw) faces(s, c, ci, cj, 0, NF);
+      p0s_interior<NG>(s, v);
+#pragma unroll
+      for (int l = 0; l < NI; ++l) {
+        if constexpr (kPacked) {
+          inter[c][l] = v[l].x;
+          inter[c + 1][l] = v[l].y;
+        } else {
+          inter[c][l] = v[l];
+        }
+      }
+    }
+    // the volume integrals of Eq. (ode2) at interior point p (weight
+    // gw[p % NG] gw[p / NG])
+    auto interior_point = [&](int p) {
+      R U[C], f[C], g[C];
+#pragma unroll
+      for (int c = 0; c < C; ++c) U[c] = inter[c][p];
+      flux(U, 0, f);
+      flux(U, 1, g);
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        Fv[c] += gw[p % NG] * gw[p / NG] * f[c];
+        Gv[c] += gw[p % NG] * gw[p / NG] * g[c];
+      }
+    };
+    if constexpr (kPacked) {  // points in pairs, an odd last one alone
+      auto flux_x2 = [&](const float2* U, int dir, float2* F) {
+        if constexpr (COMP) flux_inc2_x2(gas, B, U, dir, F);
+        else euler_flux_x2(gas, U, dir, F);
+      };
+      float2 Fv2[C], Gv2[C];
+#pragma unroll
+      for (int c = 0; c < C; ++c) Fv2[c] = Gv2[c] = make_float2(0.0f, 0.0f);
+#pragma unroll
+      for (int p = 0; p + 1 < NI; p += 2) {
+        float2 U2[C], f2[C], g2[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) U2[c] = make_float2(inter[c][p], inter[c][p + 1]);
+        flux_x2(U2, 0, f2);
+        flux_x2(U2, 1, g2);
+        const float2 w2 = make_float2(gw[p % NG] * gw[p / NG], gw[(p + 1) % NG] * gw[(p + 1) / NG]);
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          Fv2[c] = __ffma2_rn(w2, f2[c], Fv2[c]);
+          Gv2[c] = __ffma2_rn(w2, g2[c], Gv2[c]);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        Fv[c] = Fv2[c].x + Fv2[c].y;
+        Gv[c] = Gv2[c].x + Gv2[c].y;
+      }
+      if constexpr (NI % 2 == 1) interior_point(NI - 1);
+    } else {
+#pragma unroll
+      for (int p = 0; p < NI; ++p) interior_point(p);
+    }
+    list_append(&sm.nhw, sm.hwl, tid, hw, TX * TY + 2 * TX + 2 * TY);
+  }
+  for (int item = NT + tid; item < TX * TY + 2 * TX + 2 * TY; item += NT) {
+    int hi, hj, p_lo, p_hi;  // own-tile coordinates of the halo cell, point range
+    item_of(item, hi, hj, p_lo, p_hi);
+    const bool hw = near_troubled(hi, hj);
     if (!hw) {
-      // the classes of one component, or (FP32 Euler) of components c and
-      // c + 1 at once, then the face pairs the item needs
-      using T = typename PairOf<R, kPacked>::type;
 #pragma unroll
       for (int c = 0; c < C; c += kPacked ? 2 : 1) {
         T s[19];
-        classes_of<COMP, kPacked>(sm, c, ci, cj, s);
-        if (p_lo < 2 * NG) {
-          T v[2 * NG];
-          p0s_xfaces<NG>(s, v);
-#pragma unroll
-          for (int p = 0; p < 2 * NG; ++p)
-            if (p >= p_lo && p < p_hi) store_points(sm, c, p, ci, cj, v[p]);
-        }
-        if (p_hi > 2 * NG) {
-          T v[2 * NG];
-          p0s_yfaces<NG>(s, v);
-#pragma unroll
-          for (int p = 0; p < 2 * NG; ++p)
-            if (p + 2 * NG >= p_lo && p + 2 * NG < p_hi) store_points(sm, c, p + 2 * NG, ci, cj, v[p]);
-        }
+        classes_of<COMP, kPacked>(sm, c, hi, hj, s);
+        faces(s, c, hi, hj, p_lo, p_hi);
       }
     }
     list_append(&sm.nhw, sm.hwl, item, hw, TX * TY + 2 * TX + 2 * TY);
   }
   __syncthreads();
   if (sm.nhw > 0) {  // uniform over the CTA
-    for (int q = tid; q < sm.nhw; q += NT) {
+    if constexpr (C == 4 && sizeof(R) == 8) {
+      hweno_tasks_euler2d<NG, NT>(sm, sm.nhw, item_of, gam[0], gam[1], gam[2], gam[3], gam[4], eps, gas,
+                                  (a.variant & HWENO_VARIANT_MEAN_EIGEN) != 0);
+    } else for (int q = tid; q < sm.nhw; q += NT) {
       int ci, cj, p_lo, p_hi;
       item_of(sm.hwl[q], ci, cj, p_lo, p_hi);
       if constexpr (C == 1) {
@@ -673,12 +908,7 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
     __syncthreads();
   }
 
-  // ---- 4. own cells: interior points, fluxes, Eq. (ode2), Eq. (RK)
-  constexpr double r15 = 0.38729833462074168852;  // sqrt(15)/10
-  constexpr double r3 = 0.28867513459481288225;   // sqrt(3)/6
-  const R gw[3] = {NG == 3 ? R(5.0 / 18.0) : R(0.5), NG == 3 ? R(4.0 / 9.0) : R(0.5), R(5.0 / 18.0)};
-  const R gx[3] = {NG == 3 ? R(-r15) : R(-r3), NG == 3 ? R(0) : R(r3), R(r15)};
-  const int ci = ox, cj = oy;
+  // ---- 4. own cells: fluxes, Eq. (ode2), Eq. (RK)
   int myflag = 0;
   R spx = R(0), spy = R(0);
   unsigned bad = 0;
@@ -695,57 +925,12 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
     }
     myflag = sm.fl[cj + 2][ci + 2];
     const R hax = R(0.5) * alx, hay = R(0.5) * aly;
-    // COMP: every point value is an increment over the own cell's hi B, every
-    // flux an increment over f(B) (the base cancels from Eq. (ode2) exactly)
-    R B[C];
-#pragma unroll
-    for (int c = 0; c < C; ++c) B[c] = sm.u[c][0][cj + OYR][ci + OXR];
-    auto flux = [&](const R* U, int dir, R* F) {
-      if constexpr (COMP) flux_inc2<C>(gas, B, U, dir, F);
-      else phys_flux2<R, C>(gas, U, dir, F);
-    };
     // COMP: a neighbour's face value, held over its own hi, over B instead
     auto rebase = [&](R* v, int dx, int dy) {
       if constexpr (COMP) {
 #pragma unroll
         for (int c = 0; c < C; ++c)
           v[c] = __fadd_rn(v[c], __fsub_rn(sm.u[c][0][cj + OYR + dy][ci + OXR + dx], B[c]));
-      }
-    };
-    R Fv[C], Gv[C];
-#pragma unroll
-    for (int c = 0; c < C; ++c) Fv[c] = Gv[c] = R(0);
-    R inter[C][NI];
-    {
-      using T = typename PairOf<R, kPacked>::type;
-#pragma unroll
-      for (int c = 0; c < C; c += kPacked ? 2 : 1) {
-        T s[19], v[NI];
-        classes_of<COMP, kPacked>(sm, c, ci, cj, s);
-        p0s_interior<NG>(s, v);
-#pragma unroll
-        for (int l = 0; l < NI; ++l) {
-          if constexpr (kPacked) {
-            inter[c][l] = v[l].x;
-            inter[c + 1][l] = v[l].y;
-          } else {
-            inter[c][l] = v[l];
-          }
-        }
-      }
-    }
-    // the volume integrals of Eq. (ode2) at interior point p (weight
-    // gw[p % NG] gw[p / NG])
-    auto interior_point = [&](int p) {
-      R U[C], f[C], g[C];
-#pragma unroll
-      for (int c = 0; c < C; ++c) U[c] = inter[c][p];
-      flux(U, 0, f);
-      flux(U, 1, g);
-#pragma unroll
-      for (int c = 0; c < C; ++c) {
-        Fv[c] += gw[p % NG] * gw[p / NG] * f[c];
-        Gv[c] += gw[p % NG] * gw[p / NG] * g[c];
       }
     };
     R sfx[C], sfs[C], sfxe[C], sgy[C], sgs[C], sgyx[C];
@@ -810,29 +995,6 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
             v[c] = __fadd2_rn(v[c], bcast2(__fsub_rn(sm.u[c][0][cj + OYR + dy][ci + OXR + dx], B[c])));
         }
       };
-      float2 Fv2[C], Gv2[C];
-#pragma unroll
-      for (int c = 0; c < C; ++c) Fv2[c] = Gv2[c] = make_float2(0.0f, 0.0f);
-#pragma unroll
-      for (int p = 0; p + 1 < NI; p += 2) {
-        float2 U2[C], f2[C], g2[C];
-#pragma unroll
-        for (int c = 0; c < C; ++c) U2[c] = make_float2(inter[c][p], inter[c][p + 1]);
-        flux_x2(U2, 0, f2);
-        flux_x2(U2, 1, g2);
-        const float2 w2 = make_float2(gw[p % NG] * gw[p / NG], gw[(p + 1) % NG] * gw[(p + 1) / NG]);
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-          Fv2[c] = __ffma2_rn(w2, f2[c], Fv2[c]);
-          Gv2[c] = __ffma2_rn(w2, g2[c], Gv2[c]);
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < C; ++c) {
-        Fv[c] = Fv2[c].x + Fv2[c].y;
-        Gv[c] = Gv2[c].x + Gv2[c].y;
-      }
-      if constexpr (NI % 2 == 1) interior_point(NI - 1);
       float2 sfx2[C], sfs2[C], sfxe2[C], sgy2[C], sgs2[C], sgyx2[C];
 #pragma unroll
       for (int c = 0; c < C; ++c)
@@ -901,8 +1063,6 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
       if constexpr (NG % 2 == 1) face_point(NG - 1);
     } else {
 #pragma unroll
-      for (int p = 0; p < NI; ++p) interior_point(p);
-#pragma unroll
       for (int k = 0; k < NG; ++k) face_point(k);
     }
     R Uo[C];
@@ -934,7 +1094,7 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
             o[m] = rk_combine(cb, u0c[c][m], s);
           }
         }
-        if (!isfinite(o[m])) bad |= ST_NONFINITE;
+        if (!is_finite(o[m])) bad |= ST_NONFINITE;
       }
       R olo = R(0);
       if constexpr (COMP) {
@@ -1031,20 +1191,25 @@ __global__ void __launch_bounds__(NT, (sizeof(R) == 4 ? 2 : 1))
 // and leaves dt (FP64 and FP32 copies) and the last-step flag in the
 // scalars, where the three stage kernels read it.
 template <typename R>
-__global__ void __launch_bounds__(32) dt2d_kernel(const R* __restrict__ a_in, int nin,
+__global__ void __launch_bounds__(32) dt2d_kernel(const R* a_in, int nin,
                                                   DevScalars* sc, double cfl, double inv_dx,
                                                   double inv_dy) {
-  double ax = 0.0, ay = 0.0;
+  // (programmatic dependent launch on both sides: this warp is resident before
+  // the previous stage ends, and stage 1's tiles before this one does)
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const double rem = sc->rem;
+  R mx = R(0), my = R(0);  // the maxima in the kernel precision (exact), FP64 after them
   for (int k = threadIdx.x; k < nin; k += 32) {
-    ax = fmax(ax, (double)a_in[k]);
-    ay = fmax(ay, (double)a_in[nin + k]);
+    mx = fmax(mx, a_in[k]);
+    my = fmax(my, a_in[nin + k]);
   }
   for (int o = 16; o > 0; o >>= 1) {
-    ax = fmax(ax, __shfl_xor_sync(0xffffffffu, ax, o));
-    ay = fmax(ay, __shfl_xor_sync(0xffffffffu, ay, o));
+    mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    my = fmax(my, __shfl_xor_sync(0xffffffffu, my, o));
   }
   if (threadIdx.x == 0) {
-    const double rem = sc->rem;
+    const double ax = (double)mx, ay = (double)my;
     double dt = cfl / (ax * inv_dx + ay * inv_dy);
     unsigned last = 0u;
     if (rem <= 0.0) {
@@ -1061,11 +1226,11 @@ __global__ void __launch_bounds__(32) dt2d_kernel(const R* __restrict__ a_in, in
 }
 
 template <typename R, int C>
-__global__ void __launch_bounds__(NT) alpha2d_kernel(const R* __restrict__ w, R* a_out, int nx,
+__global__ void __launch_bounds__(NTW) alpha2d_kernel(const R* __restrict__ w, R* a_out, int nx,
                                                     int ny, double gas, DevScalars* sc,
                                                     int slots) {
-  __shared__ R red[2][NW];
-  const int gi = blockIdx.x * TX + threadIdx.x % TX, gj = blockIdx.y * TY + threadIdx.x / TX;
+  __shared__ R red[2][NWW];
+  const int gi = blockIdx.x * TX + threadIdx.x % TX, gj = blockIdx.y * TYW + threadIdx.x / TX;
   const size_t plane = (size_t)nx * ny;
   R sx = R(0), sy = R(0);
   if (gi < nx && gj < ny) {
@@ -1088,7 +1253,7 @@ __global__ void __launch_bounds__(NT) alpha2d_kernel(const R* __restrict__ w, R*
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int k = 0; k < NW; ++k) {
+    for (int k = 0; k < NWW; ++k) {
       sx = fmax(sx, red[0][k]);
       sy = fmax(sy, red[1][k]);
     }
@@ -1104,48 +1269,79 @@ __global__ void __launch_bounds__(NT) alpha2d_kernel(const R* __restrict__ w, R*
   }
 }
 
-template <typename R, int C, int NG, bool COMP>
-cudaError_t launch_stage2d_t(const Stage2DArgs& a0, cudaStream_t s) {
+// More than two tiles per SM: the dense build.
+bool stage2d_dense(int tiles) { return tiles > 304; }
+
+template <typename R, int C, int NG, bool COMP, bool DENSE, int TY>
+cudaError_t launch_stage2d_d(const Stage2DArgs& a0, cudaStream_t s) {
   Stage2DArgs a = a0;
   CUtensorMap map, lo_map;
-  a.tma = encode_box_map(a.w, a.nx, a.ny, 3 * C, (int)sizeof(R), RX, RY, &map) ? 1 : 0;
+  a.tma = encode_box_map(a.w, a.nx, a.ny, 3 * C, (int)sizeof(R), RX, TY + 6, &map) ? 1 : 0;
   memset(&lo_map, 0, sizeof(lo_map));
   if (COMP && a.tma)  // both boxes, or neither
-    a.tma = encode_box_map(a.w_lo, a.nx, a.ny, C, (int)sizeof(R), RX, RY, &lo_map) ? 1 : 0;
+    a.tma = encode_box_map(a.w_lo, a.nx, a.ny, C, (int)sizeof(R), RX, TY + 6, &lo_map) ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((a.nx + TX - 1) / TX), (unsigned)((a.ny + TY - 1) / TY));
-  cfg.blockDim = dim3(NT);
-  cfg.dynamicSmemBytes = sizeof(Smem2D<R, C, NG, COMP>);
+  cfg.blockDim = dim3(TX * TY);
+  cfg.dynamicSmemBytes = sizeof(Smem2D<R, C, NG, COMP, TY>);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, stage2d_kernel<R, C, NG, COMP>, a, map, lo_map);
+  return cudaLaunchKernelEx(&cfg, stage2d_kernel<R, C, NG, COMP, DENSE, TY>, a, map, lo_map);
+}
+
+// Rows of a tile: 8, or in FP64 4 (128 threads, two CTAs per SM) while the 8-row
+// tiles are a single wave: the FP64 pipes of the SMs bound those grids, and
+// half-tiles use twice as many (3 points, 4 steps, 8 / 4 rows: 40 x 40 vortex 1.67
+// / 0.98 ms, 150 x 120 1.66 / 1.22, four quadrants 3.08 / 2.35).  Beyond, smooth
+// data gain 10-20 % and data with shocks lose as much (a tile's listed items have
+// half the warps; 250 x 190 vortex 3.22 / 2.58, quadrants 3.94 / 4.42), so 8 stays.
+// FP32 is faster with 8 at every size (120 x 120 equal, 512 x 512 quadrants 11 %).
+int stage2d_rows(const Stage2DArgs& a) {
+  return a.fp64 && stage2d_tiles(a.nx, a.ny) <= 152 ? 4 : 8;
 }
 
 template <typename R, int C, int NG, bool COMP>
+cudaError_t launch_stage2d_t(const Stage2DArgs& a, cudaStream_t s) {
+  if constexpr (has_dense<R, C, NG>()) {
+    if (stage2d_dense(stage2d_tiles(a.nx, a.ny))) return launch_stage2d_d<R, C, NG, COMP, true, 8>(a, s);
+  }
+  if constexpr (sizeof(R) == 8) {
+    if (stage2d_rows(a) == 4) return launch_stage2d_d<R, C, NG, COMP, false, 4>(a, s);
+  }
+  return launch_stage2d_d<R, C, NG, COMP, false, 8>(a, s);
+}
+
+template <typename R, int C, int NG, bool COMP, bool DENSE, int TY>
 cudaError_t prepare_one() {
-  cudaError_t e = cudaFuncSetAttribute(stage2d_kernel<R, C, NG, COMP>,
+  cudaError_t e = cudaFuncSetAttribute(stage2d_kernel<R, C, NG, COMP, DENSE, TY>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sizeof(Smem2D<R, C, NG, COMP>));
+                                       (int)sizeof(Smem2D<R, C, NG, COMP, TY>));
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(stage2d_kernel<R, C, NG, COMP>,
+  return cudaFuncSetAttribute(stage2d_kernel<R, C, NG, COMP, DENSE, TY>,
                               cudaFuncAttributePreferredSharedMemoryCarveout, 100);
 }
 template <typename R, int C, int NG>
 cudaError_t prepare_t() {
-  cudaError_t e = prepare_one<R, C, NG, false>();
-  if constexpr (sizeof(R) == 4) {
-    if (e == cudaSuccess) e = prepare_one<R, C, NG, true>();
+  cudaError_t e = prepare_one<R, C, NG, false, false, 8>();
+  if constexpr (sizeof(R) == 8) {
+    if (e == cudaSuccess) e = prepare_one<R, C, NG, false, false, 4>();
+  } else {
+    if (e == cudaSuccess) e = prepare_one<R, C, NG, true, false, 8>();
+  }
+  if constexpr (has_dense<R, C, NG>()) {
+    if (e == cudaSuccess) e = prepare_one<R, C, NG, false, true, 8>();
+    if (e == cudaSuccess) e = prepare_one<R, C, NG, true, true, 8>();
   }
   return e;
 }
 
 }  // namespace
 
-int stage2d_tiles(int nx, int ny) { return ((nx + TX - 1) / TX) * ((ny + TY - 1) / TY); }
+int stage2d_tiles(int nx, int ny) { return ((nx + TX - 1) / TX) * ((ny + TYW - 1) / TYW); }
 
 bool encode_box_map(const void* w, int nx, int ny, int planes, int esize, int box_x, int box_y,
                     CUtensorMap* map) {
@@ -1217,29 +1413,38 @@ cudaError_t launch_stage2d(const Stage2DArgs& a, cudaStream_t s) {
   return a.ng == 2 ? launch_stage2d_t<float, 4, 2, false>(a, s) : launch_stage2d_t<float, 4, 3, false>(a, s);
 }
 
+template <typename R>
+static cudaError_t launch_dt2d_t(const Stage2DArgs& a, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3(32);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, dt2d_kernel<R>, static_cast<const R*>(a.a_in), a.nin, a.sc, a.cfl,
+                            a.inv_dx, a.inv_dy);
+}
+
 cudaError_t launch_dt2d(const Stage2DArgs& a, cudaStream_t s) {
-  if (a.fp64)
-    dt2d_kernel<double><<<1, 32, 0, s>>>(static_cast<const double*>(a.a_in), a.nin, a.sc, a.cfl,
-                                        a.inv_dx, a.inv_dy);
-  else
-    dt2d_kernel<float><<<1, 32, 0, s>>>(static_cast<const float*>(a.a_in), a.nin, a.sc, a.cfl,
-                                       a.inv_dx, a.inv_dy);
-  return cudaGetLastError();
+  return a.fp64 ? launch_dt2d_t<double>(a, s) : launch_dt2d_t<float>(a, s);
 }
 
 cudaError_t launch_alpha2d(const void* w, void* a_out, int nx, int ny, int system, int fp64,
                            double gas, DevScalars* sc, int slots, cudaStream_t s) {
-  dim3 grid((nx + TX - 1) / TX, (ny + TY - 1) / TY);
+  dim3 grid((nx + TX - 1) / TX, (ny + TYW - 1) / TYW);
   if (system == 0) {
     if (fp64)
-      alpha2d_kernel<double, 1><<<grid, NT, 0, s>>>(static_cast<const double*>(w), static_cast<double*>(a_out), nx, ny, gas, sc, slots);
+      alpha2d_kernel<double, 1><<<grid, NTW, 0, s>>>(static_cast<const double*>(w), static_cast<double*>(a_out), nx, ny, gas, sc, slots);
     else
-      alpha2d_kernel<float, 1><<<grid, NT, 0, s>>>(static_cast<const float*>(w), static_cast<float*>(a_out), nx, ny, gas, sc, slots);
+      alpha2d_kernel<float, 1><<<grid, NTW, 0, s>>>(static_cast<const float*>(w), static_cast<float*>(a_out), nx, ny, gas, sc, slots);
   } else {
     if (fp64)
-      alpha2d_kernel<double, 4><<<grid, NT, 0, s>>>(static_cast<const double*>(w), static_cast<double*>(a_out), nx, ny, gas, sc, slots);
+      alpha2d_kernel<double, 4><<<grid, NTW, 0, s>>>(static_cast<const double*>(w), static_cast<double*>(a_out), nx, ny, gas, sc, slots);
     else
-      alpha2d_kernel<float, 4><<<grid, NT, 0, s>>>(static_cast<const float*>(w), static_cast<float*>(a_out), nx, ny, gas, sc, slots);
+      alpha2d_kernel<float, 4><<<grid, NTW, 0, s>>>(static_cast<const float*>(w), static_cast<float*>(a_out), nx, ny, gas, sc, slots);
   }
   return cudaGetLastError();
 }

@@ -32,6 +32,28 @@ __device__ __forceinline__ R fast_sqrt(R x) {
   if constexpr (sizeof(R) == 4) return sqrt_approx(x); else return sqrt(x);
 }
 
+// x >= 0 and x > 0 without an FP64 instruction (NaN: false; -0 >= 0)
+__device__ __forceinline__ bool ge0(double x) {
+  const long long b = __double_as_longlong(x);
+  return b >= 0 ? b <= 0x7ff0000000000000ll : (b << 1) == 0;
+}
+__device__ __forceinline__ bool gt0(double x) {
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
+}
+// x truncated to FP32 by its bits (relative error < 2^-23); 0 below 2^-100,
+// NaN from 2^100 on (and for infinities and NaN): a comparison then decides
+// nothing and the FP64 form is taken.
+__device__ __forceinline__ float trunc32(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int ex = (hi >> 20) & 0x7ff;
+  unsigned b = ((unsigned)hi & 0x80000000u) | (((unsigned)(hi & 0x7fffffff) - 0x38000000u) << 3) |
+               ((unsigned)lo >> 29);
+  if (ex < 923) b = 0u;
+  if (ex >= 1123) b = 0x7fc00000u;
+  return __uint_as_float(b);
+}
+
 // bits of the device status word
 enum : unsigned { ST_NONFINITE = 1u, ST_NONPHYSICAL = 2u, ST_TIMEOUT = 4u };
 
@@ -190,10 +212,9 @@ __device__ __forceinline__ double block_max(double v, double* red) {
   return v;
 }
 
-template <typename R>
-__device__ __forceinline__ bool finite(R x) {
-  return isfinite(x);
-}
+// Finiteness; FP64 by the exponent's bits (no FP64 instruction).
+__device__ __forceinline__ bool is_finite(float x) { return isfinite(x); }
+__device__ __forceinline__ bool is_finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
 // ---------------------------------------------------------------- physics
 
