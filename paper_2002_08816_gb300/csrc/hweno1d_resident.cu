@@ -120,7 +120,11 @@ struct SmemRes {
   float mbox[CL ? 2 : 1][CL ? 6 : 1][CL ? C * NV : 1];
   float pub[CL ? 6 : 1][CL ? C * NV : 1];
   unsigned ent[CL ? 2 : 1][CL ? kMaxCluster * (NTH / 32) : 1];
-  int abort;            // a wait ran out: every thread leaves
+  // a wait ran out, every thread leaves: for a halo (set and read on either side
+  // of the cell threads' barrier), for alpha (by the scalar warp, which that
+  // barrier does not order: read only after kBarAll, or cell threads could part
+  // there, some of them waiting for the others at the next barrier)
+  int abort, abort_alpha;
   unsigned red_max[2];  // the CTA's maximum wave speed (bits), per stage parity
   unsigned arrived[2];  // warps that have folded theirs in
   unsigned trb;         // troubled cell-stages of the run
@@ -160,7 +164,7 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 && !CL ? 2 : 1) resident1
   constexpr int HS = 6 * C * NV;           // values of one CTA's published cells
 
   if (tid == 0) {
-    S.abort = 0;
+    S.abort = S.abort_alpha = 0;
     S.red_max[0] = S.red_max[1] = 0u;
     S.arrived[0] = S.arrived[1] = 0u;
     S.trb = 0u;
@@ -221,7 +225,7 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 && !CL ? 2 : 1) resident1
         if (!got) {
           if (lane == 0) {
             atomicOr(&a.sc->status, (unsigned)ST_TIMEOUT);
-            S.abort = 1;
+            S.abort_alpha = 1;
           }
           ok = false;
         }
@@ -502,7 +506,7 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 && !CL ? 2 : 1) resident1
     }
     // alpha and dt from the scalar warp
     bar_sync(kBarAll, NT + 32);
-    if (S.abort) break;
+    if (S.abort_alpha) break;
     const R alpha = sm.alpha, dt = sm.dt;
     if (!(dt > R(0))) break;  // t_final reached: uniform over the grid
 
@@ -612,7 +616,7 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 && !CL ? 2 : 1) resident1
   }
 
   // the final state, the status bits and the troubled count
-  if (own && !S.abort && done > 0) {
+  if (own && !S.abort && !S.abort_alpha && done > 0) {
     R* out = static_cast<R*>(a.out);
 #pragma unroll
     for (int c = 0; c < C; ++c) {
