@@ -55,13 +55,10 @@ constexpr int OXR = 4, OYR = 3;
 constexpr int LX = TX + 4;                // flags and modified moments, 2-cell halo
 constexpr unsigned kTmaPolls = 1u << 20;  // mbarrier polls before a tile copy is given up
 
-template <typename R, int C, int NG, bool COMP, int TY>
+template <typename R, int C, int NG, bool COMP, int TY, bool SPLIT>
 struct Smem2D {
-  static constexpr int NW = TX * TY / 32, RY = TY + 6, LY = TY + 4;
+  static constexpr int NT = TX * TY * (SPLIT ? 2 : 1), NW = NT / 32, RY = TY + 6, LY = TY + 4;
   static constexpr int kPadX = 1;  // raw index of flag-grid column lx: lx + 2
-  // the limiter's results go to `lim` by work-list slot (and are written into
-  // u once every cell's flag and limiter has read the raw moments)
-  static constexpr bool kLimList = true;
   // stage input (the TMA box); after Step 4 its first moments are the
   // modified ones
   alignas(128) R u[C][3][RY][RX];
@@ -69,9 +66,10 @@ struct Smem2D {
   alignas(128) R ulo[COMP ? C : 1][COMP ? RY : 1][COMP ? RX : 1];
   union {
     R xf[C][2 * NG][TY][TX + 2];  // x-face values (left NG, right NG) of cells -1..TX
-    R lim[C == 4 ? LX * LY : 1][C][2];  // Step 4, Euler: modified x-, y-moments by list slot
+    R lim[C == 4 ? LX * LY : 1][C][2];  // Step 4, Euler: modified x-, y-moments by list slot (into u once all have read it)
   };
   R yf[C][2 * NG][TY + 2][TX];  // y-face values (bottom NG, top NG) of cells -1..TY
+  R half[SPLIT ? 5 * C : 1][SPLIT ? TX * TY : 1];  // the second thread's sums (SPLIT)
   uint8_t fl[LY][LX];
   R red[2][NW];
   int cnt[NW];
@@ -293,111 +291,24 @@ __device__ __forceinline__ void classes_of(const S& sm, int c, int ci, int cj, T
   }
 }
 
-// Step 5.1 for an Euler cell whose 3x3 stencil holds a troubled cell: the
-// interface points [p_lo, p_hi) by HWENO in the x (x-faces) and y (y-faces)
-// characteristic fields of the cell average (Remark 4).  Rare: out of line.
-template <int NG, bool COMP, typename S, typename R>
-__device__ __noinline__ void hweno_faces_euler2d(S& sm, int ci, int cj, int p_lo, int p_hi, R g0,
-                                                 R g1, R g2, R g3, R g4, R eps, R gas,
+// Step 5.1 for the n listed Euler items, cells whose 3x3 stencil holds a troubled
+// cell: the interface points by HWENO in the x (x-faces) and y (y-faces)
+// characteristic fields of the cell average (Remark 4; mean_eigen: of the mean of
+// the two cells at each face).  (item, field) on four consecutive lanes, the two
+// directions on different warps.  An item as one thread is one chain of 2
+// directions x 4 fields, a tile's few items one warp while the rest of the SM
+// waits: in FP64, where a warp instruction takes a sub-partition 64 cycles however
+// few lanes work, ~6000 such instructions against ~550 for a task; in FP32 the
+// eigen-system and the point values of all fields also cost the kernel its
+// registers (108 bytes of spills and 1 KB of stack, none now).  FP32, an item per
+// thread -> this: 512 x 512 quadrants, 3 points, 12 steps 2.66 -> 1.38 ms; 1024 x
+// 1024 quadrants, 2 points, 12 steps 5.77 -> 3.21; 4096 x 4096 smooth, 2 points, 4
+// steps 14.7 -> 13.6; 2048 x 2048 smooth, 3 points 5.56 -> 5.07.
+template <int NG, int NT, bool COMP, typename R, typename S, typename F>
+__device__ __noinline__ void hweno_tasks_euler2d(S& sm, int n, F item_of, R g0, R g1, R g2,
+                                                 R g3, R g4, R eps, R gas,
                                                  bool mean_eigen) {
-  constexpr int NF = 4 * NG;
-  const R gam[5] = {g0, g1, g2, g3, g4};  // by value: no caller array on the stack
-  R Uc[4];
-#pragma unroll
-  for (int c = 0; c < 4; ++c) Uc[c] = sm.u[c][0][cj + OYR][ci + OXR];
-  // one eigen-system per direction (the cell average), or with mean_eigen one
-  // per face (the mean of the averages on its two sides): "parts" of the
-  // direction's 2 NG points
-  const int nparts = mean_eigen ? 2 : 1;
-#pragma unroll 1
-  for (int q = 0; q < 2 * nparts; ++q) {
-    const int dir = q / nparts, side = q % nparts;
-    const int lo = dir * 2 * NG + side * NG, hi = lo + 2 * NG / nparts;
-    const int plo = p_lo > lo ? p_lo : lo, phi = p_hi < hi ? p_hi : hi;
-    if (plo >= phi) continue;
-    R U[4];
-    if (!mean_eigen) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) U[c] = Uc[c];
-    } else {
-      const int dx = dir == 0 ? 2 * side - 1 : 0, dy = dir == 1 ? 2 * side - 1 : 0;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) U[c] = R(0.5) * (Uc[c] + sm.u[c][0][cj + OYR + dy][ci + OXR + dx]);
-    }
-    R Rm[4][4], Lm[4][4];
-    Euler2D<R>::eigen(gas, U, dir, Rm, Lm);
-    R acc[4][NF];
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int p = 0; p < NF; ++p) acc[c][p] = R(0);
-    if constexpr (sizeof(R) == 4) {
-      // FP32: the fields in pairs (f, f + 1) through the packed HWENO
-      // helpers, the stencil data of each component gathered once per pair
-#pragma unroll
-      for (int f = 0; f < 4; f += 2) {
-        float2 e2[19];
-#pragma unroll
-        for (int k = 0; k < 19; ++k) e2[k] = make_float2(0.0f, 0.0f);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          R t[19];
-          gather_data<COMP>(sm, c, ci, cj, t);
-#pragma unroll
-          for (int k = 0; k < 19; ++k) {
-            e2[k].x += Lm[f][c] * t[k];
-            e2[k].y += Lm[f + 1][c] * t[k];
-          }
-        }
-        float2 chv2[NF];
-        hweno2d_faces_x2<NG>(e2, gam, eps, plo, phi, chv2);
-#pragma unroll
-        for (int p = 0; p < NF; ++p)
-          if (p >= plo && p < phi)
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-              acc[c][p] += Rm[c][f] * chv2[p].x + Rm[c][f + 1] * chv2[p].y;
-      }
-    } else {
-#pragma unroll
-      for (int f = 0; f < 4; ++f) {
-        R e[19], t[19];
-#pragma unroll
-        for (int k = 0; k < 19; ++k) e[k] = R(0);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          gather_data<COMP>(sm, c, ci, cj, t);
-#pragma unroll
-          for (int k = 0; k < 19; ++k) e[k] += Lm[f][c] * t[k];
-        }
-        R chv[NF];
-        hweno2d_faces<NG>(e, gam, eps, plo, phi, chv);
-#pragma unroll
-        for (int p = 0; p < NF; ++p)
-          if (p >= plo && p < phi)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[c][p] += Rm[c][f] * chv[p];
-      }
-    }
-#pragma unroll
-    for (int p = 0; p < NF; ++p)
-      if (p >= plo && p < phi)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) store_point(sm, c, p, ci, cj, acc[c][p]);
-  }
-}
-
-// hweno_faces_euler2d in FP64 for the n listed items: (item, field) on four
-// consecutive lanes, the two directions on different warps.  An FP64 warp
-// instruction takes a sub-partition 64 cycles however few lanes work, and an
-// item is one long chain (2 directions x 4 fields), so a tile's few items as
-// one thread each left a single warp with ~6000 such instructions while the
-// rest of the SM waited; a task has ~550.
-template <int NG, int NT, typename S, typename F>
-__device__ __noinline__ void hweno_tasks_euler2d(S& sm, int n, F item_of, double g0, double g1, double g2,
-                                                 double g3, double g4, double eps, double gas,
-                                                 bool mean_eigen) {
-  const double gam[5] = {g0, g1, g2, g3, g4};
+  const R gam[5] = {g0, g1, g2, g3, g4};
   const int lane = threadIdx.x & 31, f = lane & 3, base = lane & ~3;
   const int dir = (threadIdx.x >> 5) & 1;
   for (int q0 = (threadIdx.x >> 6) * 8; q0 < n; q0 += NT / 64 * 8) {  // uniform over the warp
@@ -408,28 +319,28 @@ __device__ __noinline__ void hweno_tasks_euler2d(S& sm, int n, F item_of, double
       const int lo = dir * 2 * NG + side * NG, hi = lo + (mean_eigen ? NG : 2 * NG);
       const int plo = max(p_lo, lo), phi = q < n ? min(p_hi, hi) : plo;
       if (!__any_sync(0xffffffffu, plo < phi)) continue;
-      double U[4];
+      R U[4];
       const int dx = mean_eigen && dir == 0 ? 2 * side - 1 : 0, dy = mean_eigen && dir == 1 ? 2 * side - 1 : 0;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         U[c] = sm.u[c][0][cj + OYR][ci + OXR];
-        if (mean_eigen) U[c] = 0.5 * (U[c] + sm.u[c][0][cj + OYR + dy][ci + OXR + dx]);
+        if (mean_eigen) U[c] = R(0.5) * (U[c] + sm.u[c][0][cj + OYR + dy][ci + OXR + dx]);
       }
-      double Rm[4][4], Lm[4][4], l[4], r[4];
-      Euler2D<double>::eigen(gas, U, dir, Rm, Lm);
+      R Rm[4][4], Lm[4][4], l[4], r[4];
+      Euler2D<R>::eigen(gas, U, dir, Rm, Lm);
 #pragma unroll
       for (int c = 0; c < 4; ++c) {  // the row of field f; for component f, its row of Rm
         l[c] = f == 0 ? Lm[0][c] : f == 1 ? Lm[1][c] : f == 2 ? Lm[2][c] : Lm[3][c];
         r[c] = f == 0 ? Rm[0][c] : f == 1 ? Rm[1][c] : f == 2 ? Rm[2][c] : Rm[3][c];
       }
-      double e[19], ch[2 * NG];
+      R e[19], ch[2 * NG];
 #pragma unroll
-      for (int k = 0; k < 19; ++k) e[k] = 0.0;
+      for (int k = 0; k < 19; ++k) e[k] = R(0);
 #pragma unroll 1
       for (int c = 0; c < 4; ++c) {
-        double t[19];
-        const double lc = c == 0 ? l[0] : c == 1 ? l[1] : c == 2 ? l[2] : l[3];
-        gather19(sm, c, ci, cj, t);
+        R t[19];
+        const R lc = c == 0 ? l[0] : c == 1 ? l[1] : c == 2 ? l[2] : l[3];
+        gather_data<COMP>(sm, c, ci, cj, t);
 #pragma unroll
         for (int k = 0; k < 19; ++k) e[k] = fma(lc, t[k], e[k]);
       }
@@ -438,7 +349,7 @@ __device__ __noinline__ void hweno_tasks_euler2d(S& sm, int n, F item_of, double
       // component f at the points: sum over the fields, which the item's lanes hold
 #pragma unroll
       for (int p = 0; p < 2 * NG; ++p) {
-        double v = 0.0;
+        R v = R(0);
 #pragma unroll
         for (int g = 0; g < 4; ++g) v = fma(r[g], __shfl_sync(0xffffffffu, ch[p], base + g), v);
         const int pt = dir * 2 * NG + p;
@@ -451,21 +362,23 @@ __device__ __noinline__ void hweno_tasks_euler2d(S& sm, int n, F item_of, double
   }
 }
 
-// limit_euler2d in FP64 for the listed troubled cells, the same way.
-template <int NT, int LX_, typename S>
-__device__ __noinline__ void limit_tasks_euler2d(S& sm, int n, double g0, double g1, double g2, double eps,
-                                                 double gas) {
-  const double gam[3] = {g0, g1, g2};
+// Step 4 for the n listed troubled Euler cells, the same way: vbar from the
+// x-neighbours in the x characteristic fields, wbar from the y-neighbours in the y
+// fields, with the 1D Step 1 formula, to sm.lim by list slot.
+template <int NT, int LX_, typename R, typename S>
+__device__ __noinline__ void limit_tasks_euler2d(S& sm, int n, R g0, R g1, R g2, R eps,
+                                                 R gas) {
+  const R gam[3] = {g0, g1, g2};
   const int lane = threadIdx.x & 31, f = lane & 3, dir = (lane >> 2) & 1, base = lane & ~3;
   for (int q0 = (threadIdx.x >> 5) * 4; q0 < n; q0 += NT / 32 * 4) {
     const int q = q0 + (lane >> 3);
     const int k = sm.tbl[q < n ? q : q0];
     const int rx = k % LX_ + 1 + S::kPadX, ry = k / LX_ + 1;
     const int sx = dir == 0 ? 1 : 0, sy = 1 - sx, mom = 1 + dir;
-    double U[4], Rm[4][4], Lm[4][4], l[4], r[4], w[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    R U[4], Rm[4][4], Lm[4][4], l[4], r[4], w[5] = {R(0), R(0), R(0), R(0), R(0)};
 #pragma unroll
     for (int c = 0; c < 4; ++c) U[c] = sm.u[c][0][ry][rx];
-    Euler2D<double>::eigen(gas, U, dir, Rm, Lm);
+    Euler2D<R>::eigen(gas, U, dir, Rm, Lm);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       l[c] = f == 0 ? Lm[0][c] : f == 1 ? Lm[1][c] : f == 2 ? Lm[2][c] : Lm[3][c];
@@ -476,8 +389,8 @@ __device__ __noinline__ void limit_tasks_euler2d(S& sm, int n, double g0, double
       w[3] = fma(l[c], sm.u[c][mom][ry - sy][rx - sx], w[3]);
       w[4] = fma(l[c], sm.u[c][mom][ry + sy][rx + sx], w[4]);
     }
-    const double m = fld::limit_moment(w[0], w[1], w[2], w[3], w[4], gam, eps);
-    double v = 0.0;
+    const R m = fld::limit_moment(w[0], w[1], w[2], w[3], w[4], gam, eps);
+    R v = R(0);
 #pragma unroll
     for (int g = 0; g < 4; ++g) v = fma(r[g], __shfl_sync(0xffffffffu, m, base + g), v);
     if (q < n) sm.lim[q][f][dir] = v;
@@ -487,25 +400,31 @@ __device__ __noinline__ void limit_tasks_euler2d(S& sm, int n, double g0, double
 // CTAs per SM the kernel is built for.  FP32 at 128 registers holds two; where its
 // shared memory leaves room for more (Euler with 2 Gauss points: three, Burgers:
 // four), a build at 80 or 64 registers with those is the faster one on grids of
-// several waves of tiles (DENSE; 4096 x 4096 Euler, 2 points 18.7 -> 14.6 ms for 4
-// steps; 2048 x 2048 Burgers, 3 points 2.50 -> 1.63), and the slower one on a
-// single wave, which is bound by a tile's own chain (240 x 240 Euler, 2 points,
-// 30 steps 1.08 -> 1.15): stage2d_dense decides.
-template <typename R, int C, int NG, bool DENSE, int TY>
+// several waves of tiles (DENSE; 4096 x 4096 Euler, 2 points, 4 steps 18.7 -> 14.6
+// ms, 13.6 with the troubled work in tasks; 2048 x 2048 Burgers, 3 points 2.50 ->
+// 1.63), and the slower one on a single wave, which is bound by a tile's own chain
+// (240 x 240 Euler, 2 points, 30 steps 1.08 -> 1.15): stage2d_dense decides.
+template <typename R, int C, int NG, bool DENSE, int TY, bool SPLIT>
 constexpr int stage2d_ctas() {
-  return (sizeof(R) == 8 ? 1 : !DENSE ? 2 : C == 1 ? 4 : 3) * 8 / TY;
+  return SPLIT ? 1 : (sizeof(R) == 8 ? 1 : !DENSE ? 2 : C == 1 ? 4 : 3) * 8 / TY;
 }
 template <typename R, int C, int NG>
 constexpr bool has_dense() { return sizeof(R) == 4 && (C == 1 || NG == 2); }
 
-template <typename R, int C, int NG, bool COMP, bool DENSE, int TY>
-__global__ void __launch_bounds__(TX * TY, (stage2d_ctas<R, C, NG, DENSE, TY>()))
+// SPLIT: two threads per cell, for FP32 grids of at most one tile per SM (152),
+// whose stage takes as long as one tile's chain.  Step 4 and the interface items
+// take one round instead of two, a cell's second thread takes the halo items, the
+// interior points and the y-faces (its sums go to the first through shared memory).
+// 120 x 120 Euler, 3 points, 30 steps 936 -> 863 us (about half of it from the tasks above).  Beyond one tile per SM two CTAs
+// of one thread per cell overlap each other instead.
+template <typename R, int C, int NG, bool COMP, bool DENSE, int TY, bool SPLIT>
+__global__ void __launch_bounds__(TX * TY * (SPLIT ? 2 : 1), (stage2d_ctas<R, C, NG, DENSE, TY, SPLIT>()))
     stage2d_kernel(Stage2DArgs a, const __grid_constant__ CUtensorMap tile_map,
                    const __grid_constant__ CUtensorMap lo_map) {
   static_assert(!COMP || sizeof(R) == 4, "the float-pair averages are FP32");
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  using SM = Smem2D<R, C, NG, COMP, TY>;
-  constexpr int NT = TX * TY, NW = SM::NW, RY = SM::RY, LY = SM::LY;  // one own cell per thread
+  using SM = Smem2D<R, C, NG, COMP, TY, SPLIT>;
+  constexpr int NT = SM::NT, NW = SM::NW, RY = SM::RY, LY = SM::LY;
   SM& sm = *reinterpret_cast<SM*>(smem_raw);
   constexpr int NF = 4 * NG, NI = NG * NG;
   // FP32 Euler: the linear p0 maps take two components at once (packed FP32)
@@ -550,9 +469,12 @@ __global__ void __launch_bounds__(TX * TY, (stage2d_ctas<R, C, NG, DENSE, TY>())
   // dt of the step: formed in FP64 by dt2d_kernel before stage 1
   R dt_prev = R(0);
   if (a.stage > 0) dt_prev = sc_dt<R>(a.sc);
-  const int ox = tid % TX, oy = tid / TX;  // own cell of this thread
+  const int ox = tid % TX, oy = (tid / TX) % TY;  // own cell of this thread
+  // what of it this thread does (uniform over the warp): with one thread per
+  // cell everything, else the first thread faces, x-fluxes and the combination
+  const bool first = !SPLIT || tid < TX * TY, second = !SPLIT || tid >= TX * TY;
   const int gi = bx0 + ox, gj = by0 + oy;
-  const bool own = gi < nx && gj < ny;
+  const bool own = first && gi < nx && gj < ny;
   // u^n of the own cell (stages 2 and 3): brought into L2 now and loaded in
   // phase 4, so that no registers hold it through phases 2 and 3
   if (a.stage >= 2 && own) {
@@ -719,11 +641,7 @@ __global__ void __launch_bounds__(TX * TY, (stage2d_ctas<R, C, NG, DENSE, TY>())
     __syncthreads();
     tile_troubled = sm.ntb > 0;
     if (tile_troubled) {
-      if constexpr (sizeof(R) == 8) limit_tasks_euler2d<NT, LX>(sm, sm.ntb, gam[0], gam[1], gam[2], eps, gas);
-      else for (int q = tid; q < sm.ntb; q += NT) {
-        const int k = sm.tbl[q];
-        limit_euler2d(sm, k % LX, k / LX, q, gam[0], gam[1], gam[2], gam[3], gam[4], eps, gas);
-      }
+      limit_tasks_euler2d<NT, LX>(sm, sm.ntb, gam[0], gam[1], gam[2], eps, gas);
       __syncthreads();
       for (int q = tid; q < sm.ntb; q += NT) {
         const int k = sm.tbl[q];
@@ -805,13 +723,14 @@ __global__ void __launch_bounds__(TX * TY, (stage2d_ctas<R, C, NG, DENSE, TY>())
     }
   };
   {
-    const bool hw = near_troubled(ci, cj);
+    const bool hw = first && near_troubled(ci, cj);
     R inter[C][NI];
 #pragma unroll
     for (int c = 0; c < C; c += kPacked ? 2 : 1) {
       T s[19], v[NI];
       classes_of<COMP, kPacked>(sm, c, ci, cj, s);
-      if (!hw) faces(s, c, ci, cj, 0, NF);
+      if (first && !hw) faces(s, c, ci, cj, 0, NF);
+      if (!second) continue;
       p0s_interior<NG>(s, v);
 #pragma unroll
       for (int l = 0; l < NI; ++l) {
@@ -837,7 +756,8 @@ __global__ void __launch_bounds__(TX * TY, (stage2d_ctas<R, C, NG, DENSE, TY>())
         Gv[c] += gw[p % NG] * gw[p / NG] * g[c];
       }
     };
-    if constexpr (kPacked) {  // points in pairs, an odd last one alone
+    if (!second) {
+    } else if constexpr (kPacked) {  // points in pairs, an odd last one alone
       auto flux_x2 = [&](const float2* U, int dir, float2* F) {
         if constexpr (COMP) flux_inc2_x2(gas, B, U, dir, F);
         else euler_flux_x2(gas, U, dir, F);
@@ -869,9 +789,10 @@ __global__ void __launch_bounds__(TX * TY, (stage2d_ctas<R, C, NG, DENSE, TY>())
 #pragma unroll
       for (int p = 0; p < NI; ++p) interior_point(p);
     }
-    list_append(&sm.nhw, sm.hwl, tid, hw, TX * TY + 2 * TX + 2 * TY);
+    if (first) list_append(&sm.nhw, sm.hwl, tid, hw, TX * TY + 2 * TX + 2 * TY);
   }
-  for (int item = NT + tid; item < TX * TY + 2 * TX + 2 * TY; item += NT) {
+  constexpr int kItems = TX * TY + 2 * TX + 2 * TY;
+  for (int item = !SPLIT ? NT + tid : first ? kItems : tid; item < kItems; item += NT) {
     int hi, hj, p_lo, p_hi;  // own-tile coordinates of the halo cell, point range
     item_of(item, hi, hj, p_lo, p_hi);
     const bool hw = near_troubled(hi, hj);
@@ -887,22 +808,19 @@ __global__ void __launch_bounds__(TX * TY, (stage2d_ctas<R, C, NG, DENSE, TY>())
   }
   __syncthreads();
   if (sm.nhw > 0) {  // uniform over the CTA
-    if constexpr (C == 4 && sizeof(R) == 8) {
-      hweno_tasks_euler2d<NG, NT>(sm, sm.nhw, item_of, gam[0], gam[1], gam[2], gam[3], gam[4], eps, gas,
-                                  (a.variant & HWENO_VARIANT_MEAN_EIGEN) != 0);
-    } else for (int q = tid; q < sm.nhw; q += NT) {
-      int ci, cj, p_lo, p_hi;
-      item_of(sm.hwl[q], ci, cj, p_lo, p_hi);
-      if constexpr (C == 1) {
+    if constexpr (C == 4) {
+      hweno_tasks_euler2d<NG, NT, COMP>(sm, sm.nhw, item_of, gam[0], gam[1], gam[2], gam[3], gam[4], eps,
+                                        gas, (a.variant & HWENO_VARIANT_MEAN_EIGEN) != 0);
+    } else {
+      for (int q = tid; q < sm.nhw; q += NT) {
+        int ci, cj, p_lo, p_hi;
+        item_of(sm.hwl[q], ci, cj, p_lo, p_hi);
         R d[19], v[NF];
         gather_data<COMP>(sm, 0, ci, cj, d);
         hweno2d_faces<NG>(d, gam, eps, p_lo, p_hi, v);
 #pragma unroll
         for (int p = 0; p < NF; ++p)
           if (p >= p_lo && p < p_hi) store_point(sm, 0, p, ci, cj, v[p]);
-      } else {
-        hweno_faces_euler2d<NG, COMP>(sm, ci, cj, p_lo, p_hi, gam[0], gam[1], gam[2], gam[3],
-                                      gam[4], eps, gas, (a.variant & HWENO_VARIANT_MEAN_EIGEN) != 0);
       }
     }
     __syncthreads();
@@ -940,42 +858,49 @@ __global__ void __launch_bounds__(TX * TY, (stage2d_ctas<R, C, NG, DENSE, TY>())
     // weighted sums
     auto face_point = [&](int k) {
       R am[C], ap[C], fa[C], fb[C], FLk[C], FRk[C], GBk[C], GTk[C];
-      // x_{i-1/2}: u^- = right face of cell i-1, u^+ = own left face
+      if (first) {
+        // x_{i-1/2}: u^- = right face of cell i-1, u^+ = own left face
 #pragma unroll
-      for (int c = 0; c < C; ++c) { am[c] = sm.xf[c][NG + k][cj][ci]; ap[c] = sm.xf[c][k][cj][ci + 1]; }
-      rebase(am, -1, 0);
-      flux(am, 0, fa); flux(ap, 0, fb);
+        for (int c = 0; c < C; ++c) { am[c] = sm.xf[c][NG + k][cj][ci]; ap[c] = sm.xf[c][k][cj][ci + 1]; }
+        rebase(am, -1, 0);
+        flux(am, 0, fa); flux(ap, 0, fb);
 #pragma unroll
-      for (int c = 0; c < C; ++c) FLk[c] = R(0.5) * (fa[c] + fb[c]) - hax * (ap[c] - am[c]);
-      // x_{i+1/2}: u^- = own right face, u^+ = left face of cell i+1
+        for (int c = 0; c < C; ++c) FLk[c] = R(0.5) * (fa[c] + fb[c]) - hax * (ap[c] - am[c]);
+        // x_{i+1/2}: u^- = own right face, u^+ = left face of cell i+1
 #pragma unroll
-      for (int c = 0; c < C; ++c) { am[c] = sm.xf[c][NG + k][cj][ci + 1]; ap[c] = sm.xf[c][k][cj][ci + 2]; }
-      rebase(ap, 1, 0);
-      flux(am, 0, fa); flux(ap, 0, fb);
+        for (int c = 0; c < C; ++c) { am[c] = sm.xf[c][NG + k][cj][ci + 1]; ap[c] = sm.xf[c][k][cj][ci + 2]; }
+        rebase(ap, 1, 0);
+        flux(am, 0, fa); flux(ap, 0, fb);
 #pragma unroll
-      for (int c = 0; c < C; ++c) FRk[c] = R(0.5) * (fa[c] + fb[c]) - hax * (ap[c] - am[c]);
-      // y_{j-1/2}: u^- = top face of cell j-1, u^+ = own bottom face
+        for (int c = 0; c < C; ++c) FRk[c] = R(0.5) * (fa[c] + fb[c]) - hax * (ap[c] - am[c]);
 #pragma unroll
-      for (int c = 0; c < C; ++c) { am[c] = sm.yf[c][NG + k][cj][ci]; ap[c] = sm.yf[c][k][cj + 1][ci]; }
-      rebase(am, 0, -1);
-      flux(am, 1, fa); flux(ap, 1, fb);
+        for (int c = 0; c < C; ++c) {
+          sfx[c] += gw[k] * (FRk[c] - FLk[c]);
+          sfs[c] += gw[k] * (FLk[c] + FRk[c]);
+          sfxe[c] += gw[k] * gx[k] * (FRk[c] - FLk[c]);
+        }
+      }
+      if (second) {
+        // y_{j-1/2}: u^- = top face of cell j-1, u^+ = own bottom face
 #pragma unroll
-      for (int c = 0; c < C; ++c) GBk[c] = R(0.5) * (fa[c] + fb[c]) - hay * (ap[c] - am[c]);
-      // y_{j+1/2}: u^- = own top face, u^+ = bottom face of cell j+1
+        for (int c = 0; c < C; ++c) { am[c] = sm.yf[c][NG + k][cj][ci]; ap[c] = sm.yf[c][k][cj + 1][ci]; }
+        rebase(am, 0, -1);
+        flux(am, 1, fa); flux(ap, 1, fb);
 #pragma unroll
-      for (int c = 0; c < C; ++c) { am[c] = sm.yf[c][NG + k][cj + 1][ci]; ap[c] = sm.yf[c][k][cj + 2][ci]; }
-      rebase(ap, 0, 1);
-      flux(am, 1, fa); flux(ap, 1, fb);
+        for (int c = 0; c < C; ++c) GBk[c] = R(0.5) * (fa[c] + fb[c]) - hay * (ap[c] - am[c]);
+        // y_{j+1/2}: u^- = own top face, u^+ = bottom face of cell j+1
 #pragma unroll
-      for (int c = 0; c < C; ++c) GTk[c] = R(0.5) * (fa[c] + fb[c]) - hay * (ap[c] - am[c]);
+        for (int c = 0; c < C; ++c) { am[c] = sm.yf[c][NG + k][cj + 1][ci]; ap[c] = sm.yf[c][k][cj + 2][ci]; }
+        rebase(ap, 0, 1);
+        flux(am, 1, fa); flux(ap, 1, fb);
 #pragma unroll
-      for (int c = 0; c < C; ++c) {
-        sfx[c] += gw[k] * (FRk[c] - FLk[c]);
-        sfs[c] += gw[k] * (FLk[c] + FRk[c]);
-        sfxe[c] += gw[k] * gx[k] * (FRk[c] - FLk[c]);
-        sgy[c] += gw[k] * (GTk[c] - GBk[c]);
-        sgs[c] += gw[k] * (GBk[c] + GTk[c]);
-        sgyx[c] += gw[k] * gx[k] * (GTk[c] - GBk[c]);
+        for (int c = 0; c < C; ++c) GTk[c] = R(0.5) * (fa[c] + fb[c]) - hay * (ap[c] - am[c]);
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          sgy[c] += gw[k] * (GTk[c] - GBk[c]);
+          sgs[c] += gw[k] * (GBk[c] + GTk[c]);
+          sgyx[c] += gw[k] * gx[k] * (GTk[c] - GBk[c]);
+        }
       }
     };
     if constexpr (kPacked) {
@@ -1004,51 +929,59 @@ __global__ void __launch_bounds__(TX * TY, (stage2d_ctas<R, C, NG, DENSE, TY>())
         const float2 gw2 = make_float2(gw[k], gw[k + 1]);
         const float2 gwx2 = make_float2(gw[k] * gx[k], gw[k + 1] * gx[k + 1]);
         float2 am[C], ap[C], fa[C], fb[C], FL[C], FR[C], GB[C], GT[C];
+        if (first) {
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-          am[c] = make_float2(sm.xf[c][NG + k][cj][ci], sm.xf[c][NG + k + 1][cj][ci]);
-          ap[c] = make_float2(sm.xf[c][k][cj][ci + 1], sm.xf[c][k + 1][cj][ci + 1]);
+          for (int c = 0; c < C; ++c) {
+            am[c] = make_float2(sm.xf[c][NG + k][cj][ci], sm.xf[c][NG + k + 1][cj][ci]);
+            ap[c] = make_float2(sm.xf[c][k][cj][ci + 1], sm.xf[c][k + 1][cj][ci + 1]);
+          }
+          rebase_x2(am, -1, 0);
+          flux_x2(am, 0, fa); flux_x2(ap, 0, fb);
+#pragma unroll
+          for (int c = 0; c < C; ++c) FL[c] = lf_x2(fa[c], fb[c], am[c], ap[c], hax);
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            am[c] = make_float2(sm.xf[c][NG + k][cj][ci + 1], sm.xf[c][NG + k + 1][cj][ci + 1]);
+            ap[c] = make_float2(sm.xf[c][k][cj][ci + 2], sm.xf[c][k + 1][cj][ci + 2]);
+          }
+          rebase_x2(ap, 1, 0);
+          flux_x2(am, 0, fa); flux_x2(ap, 0, fb);
+#pragma unroll
+          for (int c = 0; c < C; ++c) FR[c] = lf_x2(fa[c], fb[c], am[c], ap[c], hax);
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            const float2 dx = sub2(FR[c], FL[c]);
+            sfx2[c] = __ffma2_rn(gw2, dx, sfx2[c]);
+            sfs2[c] = __ffma2_rn(gw2, __fadd2_rn(FL[c], FR[c]), sfs2[c]);
+            sfxe2[c] = __ffma2_rn(gwx2, dx, sfxe2[c]);
+          }
         }
-        rebase_x2(am, -1, 0);
-        flux_x2(am, 0, fa); flux_x2(ap, 0, fb);
+        if (second) {
 #pragma unroll
-        for (int c = 0; c < C; ++c) FL[c] = lf_x2(fa[c], fb[c], am[c], ap[c], hax);
+          for (int c = 0; c < C; ++c) {
+            am[c] = make_float2(sm.yf[c][NG + k][cj][ci], sm.yf[c][NG + k + 1][cj][ci]);
+            ap[c] = make_float2(sm.yf[c][k][cj + 1][ci], sm.yf[c][k + 1][cj + 1][ci]);
+          }
+          rebase_x2(am, 0, -1);
+          flux_x2(am, 1, fa); flux_x2(ap, 1, fb);
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-          am[c] = make_float2(sm.xf[c][NG + k][cj][ci + 1], sm.xf[c][NG + k + 1][cj][ci + 1]);
-          ap[c] = make_float2(sm.xf[c][k][cj][ci + 2], sm.xf[c][k + 1][cj][ci + 2]);
-        }
-        rebase_x2(ap, 1, 0);
-        flux_x2(am, 0, fa); flux_x2(ap, 0, fb);
+          for (int c = 0; c < C; ++c) GB[c] = lf_x2(fa[c], fb[c], am[c], ap[c], hay);
 #pragma unroll
-        for (int c = 0; c < C; ++c) FR[c] = lf_x2(fa[c], fb[c], am[c], ap[c], hax);
+          for (int c = 0; c < C; ++c) {
+            am[c] = make_float2(sm.yf[c][NG + k][cj + 1][ci], sm.yf[c][NG + k + 1][cj + 1][ci]);
+            ap[c] = make_float2(sm.yf[c][k][cj + 2][ci], sm.yf[c][k + 1][cj + 2][ci]);
+          }
+          rebase_x2(ap, 0, 1);
+          flux_x2(am, 1, fa); flux_x2(ap, 1, fb);
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-          am[c] = make_float2(sm.yf[c][NG + k][cj][ci], sm.yf[c][NG + k + 1][cj][ci]);
-          ap[c] = make_float2(sm.yf[c][k][cj + 1][ci], sm.yf[c][k + 1][cj + 1][ci]);
-        }
-        rebase_x2(am, 0, -1);
-        flux_x2(am, 1, fa); flux_x2(ap, 1, fb);
+          for (int c = 0; c < C; ++c) GT[c] = lf_x2(fa[c], fb[c], am[c], ap[c], hay);
 #pragma unroll
-        for (int c = 0; c < C; ++c) GB[c] = lf_x2(fa[c], fb[c], am[c], ap[c], hay);
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-          am[c] = make_float2(sm.yf[c][NG + k][cj + 1][ci], sm.yf[c][NG + k + 1][cj + 1][ci]);
-          ap[c] = make_float2(sm.yf[c][k][cj + 2][ci], sm.yf[c][k + 1][cj + 2][ci]);
-        }
-        rebase_x2(ap, 0, 1);
-        flux_x2(am, 1, fa); flux_x2(ap, 1, fb);
-#pragma unroll
-        for (int c = 0; c < C; ++c) GT[c] = lf_x2(fa[c], fb[c], am[c], ap[c], hay);
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-          const float2 dx = sub2(FR[c], FL[c]), dy = sub2(GT[c], GB[c]);
-          sfx2[c] = __ffma2_rn(gw2, dx, sfx2[c]);
-          sfs2[c] = __ffma2_rn(gw2, __fadd2_rn(FL[c], FR[c]), sfs2[c]);
-          sfxe2[c] = __ffma2_rn(gwx2, dx, sfxe2[c]);
-          sgy2[c] = __ffma2_rn(gw2, dy, sgy2[c]);
-          sgs2[c] = __ffma2_rn(gw2, __fadd2_rn(GB[c], GT[c]), sgs2[c]);
-          sgyx2[c] = __ffma2_rn(gwx2, dy, sgyx2[c]);
+          for (int c = 0; c < C; ++c) {
+            const float2 dy = sub2(GT[c], GB[c]);
+            sgy2[c] = __ffma2_rn(gw2, dy, sgy2[c]);
+            sgs2[c] = __ffma2_rn(gw2, __fadd2_rn(GB[c], GT[c]), sgs2[c]);
+            sgyx2[c] = __ffma2_rn(gwx2, dy, sgyx2[c]);
+          }
         }
       }
 #pragma unroll
@@ -1065,67 +998,93 @@ __global__ void __launch_bounds__(TX * TY, (stage2d_ctas<R, C, NG, DENSE, TY>())
 #pragma unroll
       for (int k = 0; k < NG; ++k) face_point(k);
     }
+    if constexpr (SPLIT) {  // the second thread's sums to the first
+      const int k = tid % (TX * TY);
+      if (second) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          sm.half[c][k] = sgy[c];
+          sm.half[C + c][k] = sgs[c];
+          sm.half[2 * C + c][k] = sgyx[c];
+          sm.half[3 * C + c][k] = Fv[c];
+          sm.half[4 * C + c][k] = Gv[c];
+        }
+      }
+      __syncthreads();
+      if (first) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          sgy[c] = sm.half[c][k];
+          sgs[c] = sm.half[C + c][k];
+          sgyx[c] = sm.half[2 * C + c][k];
+          Fv[c] = sm.half[3 * C + c][k];
+          Gv[c] = sm.half[4 * C + c][k];
+        }
+      }
+    }
     R Uo[C];
+    if (first) {
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      const R L0 = -sfx[c] * inv_dx - sgy[c] * inv_dy;
-      const R L1 = -R(0.5) * sfs[c] * inv_dx + Fv[c] * inv_dx - sgyx[c] * inv_dy;
-      const R L2 = -sfxe[c] * inv_dx - R(0.5) * sgs[c] * inv_dy + Gv[c] * inv_dy;
-      // the stage input the combination uses: first moments as modified by
-      // Step 4 (stored, the default), or unmodified (variant)
-      // (the tile holds the modified ones; the raw ones of an own cell are
-      // read back from the stage input)
-      const bool raw = (a.variant & HWENO_VARIANT_RAW_COMBINE) != 0;
-      const size_t sw = (size_t)gj * nx + gi;
-      const R W[3] = {sm.u[c][0][cj + OYR][ci + OXR],
-                      raw ? (own ? w[(3 * c + 1) * plane + sw] : R(0)) : sm.u[c][1][cj + OYR][ci + OXR],
-                      raw ? (own ? w[(3 * c + 2) * plane + sw] : R(0)) : sm.u[c][2][cj + OYR][ci + OXR]};
-      const R Lm[3] = {L0, L1, L2};
-      R o[3];
+      for (int c = 0; c < C; ++c) {
+        const R L0 = -sfx[c] * inv_dx - sgy[c] * inv_dy;
+        const R L1 = -R(0.5) * sfs[c] * inv_dx + Fv[c] * inv_dx - sgyx[c] * inv_dy;
+        const R L2 = -sfxe[c] * inv_dx - R(0.5) * sgs[c] * inv_dy + Gv[c] * inv_dy;
+        // the stage input the combination uses: first moments as modified by
+        // Step 4 (stored, the default), or unmodified (variant)
+        // (the tile holds the modified ones; the raw ones of an own cell are
+        // read back from the stage input)
+        const bool raw = (a.variant & HWENO_VARIANT_RAW_COMBINE) != 0;
+        const size_t sw = (size_t)gj * nx + gi;
+        const R W[3] = {sm.u[c][0][cj + OYR][ci + OXR],
+                        raw ? (own ? w[(3 * c + 1) * plane + sw] : R(0)) : sm.u[c][1][cj + OYR][ci + OXR],
+                        raw ? (own ? w[(3 * c + 2) * plane + sw] : R(0)) : sm.u[c][2][cj + OYR][ci + OXR]};
+        const R Lm[3] = {L0, L1, L2};
+        R o[3];
 #pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        if (a.stage == 0) {
-          o[m] = Lm[m];
-        } else {
-          const R s = W[m] + dt * Lm[m];
-          if (a.stage == 1) o[m] = s;
-          else {
-            const R cb = a.stage == 2 ? R(0.25) : R(2.0 / 3.0);
-            o[m] = rk_combine(cb, u0c[c][m], s);
+        for (int m = 0; m < 3; ++m) {
+          if (a.stage == 0) {
+            o[m] = Lm[m];
+          } else {
+            const R s = W[m] + dt * Lm[m];
+            if (a.stage == 1) o[m] = s;
+            else {
+              const R cb = a.stage == 2 ? R(0.25) : R(2.0 / 3.0);
+              o[m] = rk_combine(cb, u0c[c][m], s);
+            }
+          }
+          if (!is_finite(o[m])) bad |= ST_NONFINITE;
+        }
+        R olo = R(0);
+        if constexpr (COMP) {
+          // the average as a float pair: a u^n + b w in pair arithmetic (1/3
+          // and 2/3 as pairs), then the increment b dt L
+          constexpr float t1h = 1.0f / 3.0f, t2h = 2.0f / 3.0f;
+          constexpr float t1l = (float)(1.0 / 3.0 - (double)t1h), t2l = (float)(2.0 / 3.0 - (double)t2h);
+          const R wl = sm.ulo[c][cj + OYR][ci + OXR];
+          R bh = W[0], bl = wl;
+          if (a.stage == 2)
+            pair_axpby(0.75f, 0.0f, u0c[c][0], u0l[c], 0.25f, 0.0f, W[0], wl, bh, bl);
+          else if (a.stage == 3)
+            pair_axpby(t1h, t1l, u0c[c][0], u0l[c], t2h, t2l, W[0], wl, bh, bl);
+          const R cb = a.stage == 2 ? R(0.25) : a.stage == 3 ? R(2.0 / 3.0) : R(1);
+          pair_add(bh, bl, (cb * dt) * L0, o[0], olo);
+          if (!isfinite(o[0])) bad |= ST_NONFINITE;
+        }
+        if (own) {
+          R* out = static_cast<R*>(a.out);
+          const size_t s = (size_t)gj * nx + gi;
+#pragma unroll
+          for (int m = 0; m < 3; ++m) out[(3 * c + m) * plane + s] = o[m];
+          if constexpr (COMP) a.out_lo[c * plane + s] = olo;
+          if (a.lim_out) {  // rhs mode: the modified moments; stage 1: what stages 2-3 combine
+            R* lo = static_cast<R*>(a.lim_out);
+            const R M[3] = {W[0], sm.u[c][1][cj + OYR][ci + OXR], sm.u[c][2][cj + OYR][ci + OXR]};
+#pragma unroll
+            for (int m = 0; m < 3; ++m) lo[(3 * c + m) * plane + s] = a.stage == 0 ? M[m] : W[m];
           }
         }
-        if (!is_finite(o[m])) bad |= ST_NONFINITE;
+        Uo[c] = o[0];
       }
-      R olo = R(0);
-      if constexpr (COMP) {
-        // the average as a float pair: a u^n + b w in pair arithmetic (1/3
-        // and 2/3 as pairs), then the increment b dt L
-        constexpr float t1h = 1.0f / 3.0f, t2h = 2.0f / 3.0f;
-        constexpr float t1l = (float)(1.0 / 3.0 - (double)t1h), t2l = (float)(2.0 / 3.0 - (double)t2h);
-        const R wl = sm.ulo[c][cj + OYR][ci + OXR];
-        R bh = W[0], bl = wl;
-        if (a.stage == 2)
-          pair_axpby(0.75f, 0.0f, u0c[c][0], u0l[c], 0.25f, 0.0f, W[0], wl, bh, bl);
-        else if (a.stage == 3)
-          pair_axpby(t1h, t1l, u0c[c][0], u0l[c], t2h, t2l, W[0], wl, bh, bl);
-        const R cb = a.stage == 2 ? R(0.25) : a.stage == 3 ? R(2.0 / 3.0) : R(1);
-        pair_add(bh, bl, (cb * dt) * L0, o[0], olo);
-        if (!isfinite(o[0])) bad |= ST_NONFINITE;
-      }
-      if (own) {
-        R* out = static_cast<R*>(a.out);
-        const size_t s = (size_t)gj * nx + gi;
-#pragma unroll
-        for (int m = 0; m < 3; ++m) out[(3 * c + m) * plane + s] = o[m];
-        if constexpr (COMP) a.out_lo[c * plane + s] = olo;
-        if (a.lim_out) {  // rhs mode: the modified moments; stage 1: what stages 2-3 combine
-          R* lo = static_cast<R*>(a.lim_out);
-          const R M[3] = {W[0], sm.u[c][1][cj + OYR][ci + OXR], sm.u[c][2][cj + OYR][ci + OXR]};
-#pragma unroll
-          for (int m = 0; m < 3; ++m) lo[(3 * c + m) * plane + s] = a.stage == 0 ? M[m] : W[m];
-        }
-      }
-      Uo[c] = o[0];
     }
     if (own) {
       if (a.flags_out) a.flags_out[(size_t)gj * nx + gi] = (uint8_t)myflag;
@@ -1272,7 +1231,7 @@ __global__ void __launch_bounds__(NTW) alpha2d_kernel(const R* __restrict__ w, R
 // More than two tiles per SM: the dense build.
 bool stage2d_dense(int tiles) { return tiles > 304; }
 
-template <typename R, int C, int NG, bool COMP, bool DENSE, int TY>
+template <typename R, int C, int NG, bool COMP, bool DENSE, int TY, bool SPLIT = false>
 cudaError_t launch_stage2d_d(const Stage2DArgs& a0, cudaStream_t s) {
   Stage2DArgs a = a0;
   CUtensorMap map, lo_map;
@@ -1282,15 +1241,15 @@ cudaError_t launch_stage2d_d(const Stage2DArgs& a0, cudaStream_t s) {
     a.tma = encode_box_map(a.w_lo, a.nx, a.ny, C, (int)sizeof(R), RX, TY + 6, &lo_map) ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((a.nx + TX - 1) / TX), (unsigned)((a.ny + TY - 1) / TY));
-  cfg.blockDim = dim3(TX * TY);
-  cfg.dynamicSmemBytes = sizeof(Smem2D<R, C, NG, COMP, TY>);
+  cfg.blockDim = dim3(Smem2D<R, C, NG, COMP, TY, SPLIT>::NT);
+  cfg.dynamicSmemBytes = sizeof(Smem2D<R, C, NG, COMP, TY, SPLIT>);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, stage2d_kernel<R, C, NG, COMP, DENSE, TY>, a, map, lo_map);
+  return cudaLaunchKernelEx(&cfg, stage2d_kernel<R, C, NG, COMP, DENSE, TY, SPLIT>, a, map, lo_map);
 }
 
 // Rows of a tile: 8, or in FP64 4 (128 threads, two CTAs per SM) while the 8-row
@@ -1311,17 +1270,19 @@ cudaError_t launch_stage2d_t(const Stage2DArgs& a, cudaStream_t s) {
   }
   if constexpr (sizeof(R) == 8) {
     if (stage2d_rows(a) == 4) return launch_stage2d_d<R, C, NG, COMP, false, 4>(a, s);
+  } else {
+    if (stage2d_tiles(a.nx, a.ny) <= 152) return launch_stage2d_d<R, C, NG, COMP, false, 8, true>(a, s);
   }
   return launch_stage2d_d<R, C, NG, COMP, false, 8>(a, s);
 }
 
-template <typename R, int C, int NG, bool COMP, bool DENSE, int TY>
+template <typename R, int C, int NG, bool COMP, bool DENSE, int TY, bool SPLIT = false>
 cudaError_t prepare_one() {
-  cudaError_t e = cudaFuncSetAttribute(stage2d_kernel<R, C, NG, COMP, DENSE, TY>,
+  cudaError_t e = cudaFuncSetAttribute(stage2d_kernel<R, C, NG, COMP, DENSE, TY, SPLIT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sizeof(Smem2D<R, C, NG, COMP, TY>));
+                                       (int)sizeof(Smem2D<R, C, NG, COMP, TY, SPLIT>));
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(stage2d_kernel<R, C, NG, COMP, DENSE, TY>,
+  return cudaFuncSetAttribute(stage2d_kernel<R, C, NG, COMP, DENSE, TY, SPLIT>,
                               cudaFuncAttributePreferredSharedMemoryCarveout, 100);
 }
 template <typename R, int C, int NG>
@@ -1331,6 +1292,8 @@ cudaError_t prepare_t() {
     if (e == cudaSuccess) e = prepare_one<R, C, NG, false, false, 4>();
   } else {
     if (e == cudaSuccess) e = prepare_one<R, C, NG, true, false, 8>();
+    if (e == cudaSuccess) e = prepare_one<R, C, NG, false, false, 8, true>();
+    if (e == cudaSuccess) e = prepare_one<R, C, NG, true, false, 8, true>();
   }
   if constexpr (has_dense<R, C, NG>()) {
     if (e == cudaSuccess) e = prepare_one<R, C, NG, false, true, 8>();
