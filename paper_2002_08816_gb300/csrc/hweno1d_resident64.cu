@@ -17,9 +17,9 @@
 //
 // Measured (GB300, one pass of set_state, steps, get_state, before: per-stage or
 // persistent launches with a cell per thread): 400 cells with shocks, 60 steps
-// 9.57 -> 2.84 ms (15.6 us per stage); 65536 cells, 10 steps 2.33 -> 1.14 ms
-// (37 us per stage; the FP64 instructions alone would take ~26).  One CTA of 432
-// cells per SM instead of two of 216: 1.27 ms.
+// 9.57 -> 2.86 ms (15.9 us per stage); 65536 cells, 10 steps 2.33 -> 1.20 ms
+// (40 us per stage; the FP64 instructions alone would take ~28).  One CTA of 432
+// cells per SM instead of two of 216: 12 % slower.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

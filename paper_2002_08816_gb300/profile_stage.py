@@ -15,7 +15,8 @@ EVERY (2D) the steps are recorded with a checkpoint every EVERY steps and the
 gradient of sum(rho^2) is taken (hweno_backward: recomputed stages, then two
 adjoint kernels per stage).  With --batch N it runs N independent 1D Euler
 instances in shared launches (hweno_create_batch).  --persistent and
---resident select the 1D launch kinds with one launch per run.  --quadrants
+--resident select the 1D launch kinds with one launch per run (a single instance
+whose tiles fit on the GPU at once runs resident under every choice).  --quadrants
 (2D) replaces the vortex by four constant quadrants drawn from the seed (shocks
 along the quadrant lines: the troubled-cell paths); --lax-tiles (1D Euler)
 replaces the two-state data by Lax's Riemann problem repeated every 800 cells
@@ -50,7 +51,7 @@ def main():
     ap.add_argument("--threads", type=int, default=0, choices=[0, 128, 256, 512],
                     help="1D: threads per CTA (0: the default)")
     ap.add_argument("--persistent", action="store_true",
-                    help="1D: one persistent launch with grid barriers instead of per-stage graphs")
+                    help="1D FP64 grids too large to stay on chip: one persistent launch")
     ap.add_argument("--resident", action="store_true",
                     help="1D FP32: one resident launch (tiles kept on chip) per run")
     ap.add_argument("--quadrants", action="store_true",
