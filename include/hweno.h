@@ -238,8 +238,9 @@ hweno_status hweno_rhs_vjp(hweno_handle h, const void* in, const uint8_t* flags,
  * restored afterwards.  The paper has no counterpart (it fixes no hardware
  * mapping).  choice_out (nullable, 2 ints) receives the threads per CTA and the
  * launch kind (0 graphs, 1 persistent, 2 resident).  New handles start with 256
- * threads and kind 0 (HWENO_FP32C: kind 2, the only one it has; its autotuner
- * times 256 and 512 threads).  Waits for the stream; HWENO_ERR_ARG for 2D
+ * threads and kind 0 (HWENO_FP32C: kind 2, the only one it has).  A single FP32
+ * or HWENO_FP32C instance that runs resident under every choice is timed with 256
+ * and 512 threads of kind 2.  Waits for the stream; HWENO_ERR_ARG for 2D
  * handles, HWENO_ERR_STATE before set_state. */
 hweno_status hweno_autotune(hweno_handle h, int nsteps_trial, int* choice_out);
 

@@ -1331,8 +1331,16 @@ hweno_status hweno_autotune(hweno_handle h, int nsteps_trial, int* choice_out) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
-  for (int persist = h->comp ? 2 : 0; persist < 3 && e == cudaSuccess; ++persist)
-    for (int ci = h->comp ? 1 : 0; ci < 3 && e == cudaSuccess; ++ci) {
+  // an FP32 instance that runs resident under every choice has only that launch's
+  // threads to choose (the others would time the same run)
+  bool res_only = h->comp;
+  if (e == cudaSuccess && !res_only && h->n_batch == 0 && h->esize == 4) {
+    e = prepare_resident(h, 256);
+    res_only = e == cudaSuccess && h->res_tile > 0;
+  }
+  for (int persist = res_only ? 2 : 0; persist < 3 && e == cudaSuccess; ++persist) {
+    if (persist == 1 && h->esize == 4) continue;  // FP32: the per-stage launches again
+    for (int ci = res_only ? 1 : 0; ci < 3 && e == cudaSuccess; ++ci) {
       e = configure(cand_nth[ci], persist);
       if (e != cudaSuccess) break;
       if (persist == 2 && h->res_tile == 0) continue;  // not available here
@@ -1366,6 +1374,7 @@ hweno_status hweno_autotune(hweno_handle h, int nsteps_trial, int* choice_out) {
         best_persist = persist;
       }
     }
+  }
   if (e == cudaSuccess) e = configure(best_nth, best_persist);
   if (e == cudaSuccess) e = copy_all(false);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
