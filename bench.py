@@ -57,12 +57,12 @@ TRAFFIC_1D_FP32C = {(256, "resident"): (2937856 + 55808) / 6000}
 TRAFFIC_TROUBLED_1D = {(256, "resident"): (1767936 + 53248) / 600}
 # the batched workload, 128-thread per-stage launches: the mean of the three
 # stages of one step, cold L2
-TRAFFIC_BATCH_FP32 = {(128, "per-stage graphs"): (48942336 + 43494656 + 96712960 + 22568192
-                                                  + 96711424 + 21799936) / 3}
+TRAFFIC_BATCH_FP32 = {(128, "per-stage graphs"): (48290048 + 35837952 + 96035328 + 14390528
+                                                  + 96035840 + 14393344) / 3}
 # 2D, 2 Gauss points: a 2048^2 capture (the three stages of one step) scaled
 # by the cell count to 4096^2 (the bytes per cell do not depend on the grid)
-TRAFFIC_2D_NG2 = 4 * (202326016 + 350454528 + 403358976 + 173675008 + 403536384
-                      + 175169536) / 3
+TRAFFIC_2D_NG2 = 4 * (201989888 + 347983872 + 403423744 + 172841472 + 403365632
+                      + 174379008) / 3
 L2_FLUSH_BYTES = 512 << 20
 # hweno_autotune's launch kinds and the kernel each one times
 LAUNCH_KIND = {0: "per-stage graphs", 1: "persistent", 2: "resident"}
@@ -309,6 +309,7 @@ def run_1d(H, s, stream, u0, prec, steps, warmup, flush, sampler=None, autotune=
     # this workload (untimed)
     H.hweno_set_state(h, dev_in.data_ptr(), sdt, True)
     choice = H.hweno_autotune(h, 100) if autotune else (256, 0)
+    choice = (choice[0], 2)  # this grid runs resident under every choice, FP64 too
     for _ in range(warmup):
         one_step()
     torch.cuda.synchronize()
