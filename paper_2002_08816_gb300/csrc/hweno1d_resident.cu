@@ -534,8 +534,14 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 && !CL ? 2 : 1) resident1
           ov = sv;
         } else {
           const R cb = stage == 2 ? R(0.25) : R(2.0 / 3.0);
-          ou = rk_combine(cb, u0c[c][0], su);
-          ov = rk_combine(cb, u0c[c][1], sv);
+          if constexpr (CL && !COMP) {
+            const R ca = stage == 2 ? R(0.75) : R(1.0 / 3.0);
+            ou = rk_printed(ca, cb, u0c[c][0], su);
+            ov = rk_printed(ca, cb, u0c[c][1], sv);
+          } else {
+            ou = rk_combine(cb, u0c[c][0], su);
+            ov = rk_combine(cb, u0c[c][1], sv);
+          }
         }
         if constexpr (COMP) {
           // the averages: the pair formed before alpha plus the stage's increment

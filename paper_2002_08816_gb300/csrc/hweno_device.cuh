@@ -99,6 +99,16 @@ template <typename R>
 __device__ __forceinline__ R rk_combine(R b, R z, R s) {
   return fma(b, s - z, z);
 }
+// The printed form, for the FP32 cluster runs (grids of up to about 4000 cells):
+// on a shock tube of a few hundred cells some KXRCF indicators come so close to the
+// threshold that the rounding of the combination decides them, and these grids keep
+// the results, bit for bit, of their per-stage launches (so the order of the two
+// products is spelled out).  Lax's tube, 200 cells, 60 steps, 120 inputs, against 64
+// bits: here 9.7e-7 at the median and one input decided otherwise (1.9e-5); with
+// rk_combine 2.2e-7 and four (up to 3.0e-4).
+__device__ __forceinline__ float rk_printed(float a, float b, float z, float s) {
+  return fmaf(a, z, __fmul_rn(b, s));
+}
 
 // Ghost cells: periodic wraps, outflow copies the boundary cell.  Any g
 // (a tile's halo may span several periods when n is smaller than a tile).
