@@ -50,6 +50,7 @@ using s1d::ConsVec;
 using s1d::H;
 using s1d::kBarAll;
 using s1d::kBarCells;
+using s1d::kBarTaken;
 using s1d::ldx;
 using s1d::Smem1D;
 
@@ -122,8 +123,9 @@ struct SmemRes {
   unsigned ent[CL ? 2 : 1][CL ? kMaxCluster * (NTH / 32) : 1];
   // a wait ran out, every thread leaves: for a halo (set and read on either side
   // of the cell threads' barrier), for alpha (by the scalar warp, which that
-  // barrier does not order: read only after kBarAll, or cell threads could part
-  // there, some of them waiting for the others at the next barrier)
+  // barrier does not order: written between kBarTaken and kBarAll and read after
+  // kBarAll, or cell threads could part there, some of them waiting for the others
+  // at the next barrier)
   int abort, abort_alpha;
   unsigned red_max[2];  // the CTA's maximum wave speed (bits), per stage parity
   unsigned arrived[2];  // warps that have folded theirs in
@@ -222,14 +224,21 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 && !CL ? 2 : 1) resident1
           got = tag_of(w) == (unsigned)s;
           m = value_of(w);
         }
-        if (!got) {
-          if (lane == 0) {
+        ok = got;
+        alpha = (double)m;
+        if constexpr (!CL) {
+          // not before the cell threads have read stage s - 1's alpha, dt and flag
+          // (a wait may run out long before they do: written over, or with a second
+          // arrival on kBarAll before theirs, some of them would go on and wait for
+          // the others for ever), or have left
+          __syncwarp();
+          bar_sync(kBarTaken, NT + 32);
+          if (S.abort) ok = false;
+          if (!ok && lane == 0) {
             atomicOr(&a.sc->status, (unsigned)ST_TIMEOUT);
             S.abort_alpha = 1;
           }
-          ok = false;
         }
-        alpha = (double)m;
       }
       if (stage == 1) {
         dt = a.cfl_dx / alpha;
@@ -257,6 +266,9 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 && !CL ? 2 : 1) resident1
         ++done_steps;
       }
       if constexpr (CL) cluster_meet(ncta);
+    }
+    if constexpr (!CL) {
+      if (ok) bar_sync(kBarTaken, NT + 32);  // (the last arrival there)
     }
     // alpha of the final state for the next call (slot 0 of the first
     // buffer, the other slots and the second buffer zero, as the per-stage
@@ -400,7 +412,11 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 && !CL ? 2 : 1) resident1
       }
     }
     bar_sync(kBarCells, NT);
-    if (S.abort) break;
+    if (S.abort) {  // leave, past the barriers the scalar warp counts on
+      bar_sync(kBarAll, NT + 32);
+      bar_arrive(kBarTaken, NT + 32);
+      break;
+    }
     if (s == 0 && own) {
 #pragma unroll
       for (int c = 0; c < C; ++c) {
@@ -508,6 +524,7 @@ __global__ void __launch_bounds__(NTH + 32, NTH == 256 && !CL ? 2 : 1) resident1
     bar_sync(kBarAll, NT + 32);
     if (S.abort_alpha) break;
     const R alpha = sm.alpha, dt = sm.dt;
+    if constexpr (!CL) bar_arrive(kBarTaken, NT + 32);
     if (!(dt > R(0))) break;  // t_final reached: uniform over the grid
 
     // the Runge-Kutta combination; the output stays in registers, the first

@@ -38,6 +38,7 @@ using s1d::bar_sync;
 using s1d::H;
 using s1d::kBarAll;
 using s1d::kBarCells;
+using s1d::kBarTaken;
 using s1d::ldx;
 
 __device__ __forceinline__ void publish(u64* dst, unsigned tag, double v) {
@@ -89,8 +90,8 @@ struct SmemRes64 {
   Smem64<C, TMAX> w;
   double u0[C][2][TMAX];  // u^n as limited by stage 1
   // a wait ran out, every thread leaves: set by a halo thread and read after
-  // the barrier that opens a stage, or by the scalar warp and read after the
-  // one that brings alpha (two flags, so that all threads see the same)
+  // the barrier that opens a stage, or by the scalar warp, between kBarTaken and
+  // kBarAll, and read after kBarAll (two flags, so that all threads see the same)
   int abort, abort_alpha;
   unsigned arrived[2];    // warps that have folded their wave speeds in, by stage parity
   u64 red_max[2];
@@ -148,6 +149,13 @@ __global__ void __launch_bounds__(NTH + 32, 2) resident64_kernel(Resident1DArgs 
       } else {
         ok = gather_max64<1>(r.alpha_word + 2 * ((s - 1) & 1), 1, (unsigned)s, lane, &alpha, r.polls);
       }
+      if (s > 0) {
+        // not before the cell threads have read stage s - 1's alpha, dt and flag, or
+        // have left (as in the FP32 run)
+        __syncwarp();
+        bar_sync(kBarTaken, NTH + 32);
+        if (S.abort) ok = false;
+      }
       if (!ok && lane == 0) {
         atomicOr(&a.sc->status, (unsigned)ST_TIMEOUT);
         S.abort_alpha = 1;
@@ -178,6 +186,7 @@ __global__ void __launch_bounds__(NTH + 32, 2) resident64_kernel(Resident1DArgs 
         ++done_steps;
       }
     }
+    if (ok) bar_sync(kBarTaken, NTH + 32);  // (the last arrival there)
     // alpha of the final state for the next call, as the per-stage launches
     // leave it, once every CTA has published its last stage
     if (q == 0 && ok && s_end > 0) {
@@ -262,12 +271,17 @@ __global__ void __launch_bounds__(NTH + 32, 2) resident64_kernel(Resident1DArgs 
       }
     }
     bar_sync(kBarCells, NTH);
-    if (S.abort) break;
+    if (S.abort) {  // leave, past the barriers the scalar warp counts on
+      bar_sync(kBarAll, NTH + 32);
+      bar_arrive(kBarTaken, NTH + 32);
+      break;
+    }
     const int mine = f64::step1<C, TMAX, NTH>(sm, u, Tq, tid, par);
     f64::step2<C, TMAX, NTH>(sm, u, Tq, tid, par);
     bar_sync(kBarAll, NTH + 32);  // alpha and dt from the scalar warp
     if (S.abort_alpha) break;
     const double alpha = sm.alpha, dt = sm.dt;
+    bar_arrive(kBarTaken, NTH + 32);
     if (!(dt > 0.0)) break;  // t_final reached: uniform over the grid
     trb += mine;
     f64::lax_friedrichs<C, TMAX, NTH>(sm, Tq, tid, alpha);

@@ -44,8 +44,10 @@ namespace s1d {
 constexpr int H = 3;  // halo cells per side
 
 // Named barriers: kBarCells among the NTH cell threads only; kBarAll for the
-// cell threads and the scalar warp (which only arrives) before step 4.
-constexpr int kBarCells = 1, kBarAll = 2;
+// cell threads and the scalar warp (which only arrives) before step 4; kBarTaken
+// (resident runs) for the cell threads, which arrive once they have read alpha and
+// dt, and the scalar warp, which waits there before it writes the next ones.
+constexpr int kBarCells = 1, kBarAll = 2, kBarTaken = 3;
 __device__ __forceinline__ void bar_sync(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
