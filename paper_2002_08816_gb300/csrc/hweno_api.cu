@@ -356,6 +356,19 @@ cudaError_t enqueue_resident1d(hweno_ctx* h, int nsteps, cudaStream_t s, int sil
   return hw::launch_resident1d(r, h->res_nth, h->res_ncta, s);
 }
 
+// nsteps steps as launches of at most 2^29 (a resident run counts its stages in 32
+// bits); once t_final is reached a launch ends at its first stage.
+template <typename F>
+cudaError_t in_launches(int nsteps, F launch) {
+  constexpr int kMost = 1 << 29;
+  for (; nsteps > 0; nsteps -= kMost) {
+    const cudaError_t e = launch(nsteps < kMost ? nsteps : kMost);
+    if (e != cudaSuccess) return e;
+    if (nsteps <= kMost) break;
+  }
+  return cudaSuccess;
+}
+
 // nsteps Runge-Kutta steps of a small FP32 or float-pair handle in one launch
 // of one cluster.
 cudaError_t enqueue_cluster1d(hweno_ctx* h, int nsteps, cudaStream_t s) {
@@ -782,14 +795,14 @@ hweno_status hweno_step(hweno_handle h, int nsteps, double t_final, double* t_ou
     // FP32 grids that fit one cluster run there, whatever launch the handle is
     // set to: a stage is then bound by its own latency and not by a launch or a
     // round trip to L2 (Lax on 200 cells: 3.7 us per stage by launches, 2.35 on chip)
-    HW_CUDA(h, enqueue_cluster1d(h, left, h->stream));
+    HW_CUDA(h, in_launches(left, [&](int k) { return enqueue_cluster1d(h, k, h->stream); }));
     left = 0;
   }
   if (h->tile64 > 0 && h->n_batch == 0 && left > 0) {
     // FP64 single instances whose tiles fit on the GPU at once run on chip,
     // whatever launch the handle is set to: at every size the FP64 pipe and not
     // the launches bounds them, and the resident run spreads it best
-    cudaError_t e = enqueue_resident64(h, left, h->stream);
+    cudaError_t e = in_launches(left, [&](int k) { return enqueue_resident64(h, k, h->stream); });
     if (e == cudaSuccess) {
       left = 0;
     } else if (e == cudaErrorCooperativeLaunchTooLarge) {
@@ -806,7 +819,7 @@ hweno_status hweno_step(hweno_handle h, int nsteps, double t_final, double* t_ou
     const int nth = h->persist1d == 2 ? h->nth1d : 256;
     if (h->res_nth != nth) HW_CUDA(h, prepare_resident(h, nth));
     if (h->res_tile > 0) {
-      cudaError_t e = enqueue_resident1d(h, left, h->stream);
+      cudaError_t e = in_launches(left, [&](int k) { return enqueue_resident1d(h, k, h->stream); });
       if (e == cudaErrorCooperativeLaunchTooLarge && h->persist1d != 2) {
         cudaGetLastError();
         h->res_tile = 0;
@@ -1433,7 +1446,7 @@ hweno_status hweno_check_resident(hweno_handle h, int nsteps, int silent_cta, un
                 "hweno_check_resident: need nsteps >= 1, -1 <= silent_cta < CTAs, polls >= 1");
   if (h->res_nth != h->nth1d) HW_CUDA(h, prepare_resident(h, h->nth1d));
   HW_CUDA(h, hw::launch_set_scalars(h->sc, 0, -1.0, h->stream));
-  HW_CUDA(h, enqueue_resident1d(h, nsteps, h->stream, silent_cta, polls));
+  HW_CUDA(h, in_launches(nsteps, [&](int k) { return enqueue_resident1d(h, k, h->stream, silent_cta, polls); }));
   hw::DevScalars host;
   return check_scalars(h, h->sc, &host);  // HWENO_ERR_TIMEOUT when a wait ran out
 }
