@@ -796,11 +796,9 @@ size_t resident1d_halo_words(int system, int ncta) {
   return (size_t)ncta * 2 * 6 * (system == 0 ? 1 : 3) * 3;
 }
 
-cudaError_t launch_resident1d(const Resident1DArgs& r, int nth, int ncta, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(r.halo, 0,
-                                  sizeof(unsigned long long) * resident1d_halo_words(r.a.system, ncta), s);
-  if (e == cudaSuccess)
-    e = cudaMemsetAsync(r.entries, 0, sizeof(unsigned long long) * resident1d_entry_words(ncta), s);
+cudaError_t launch_resident1d(const Resident1DArgs& r, int nth, int ncta, double t_final, cudaStream_t s) {
+  const cudaError_t e = launch_start_run(r.a.sc, t_final, r.halo, resident1d_halo_words(r.a.system, ncta),
+                                         r.entries, resident1d_entry_words(ncta), s);
   if (e != cudaSuccess) return e;
   return resident_dispatch(r.a.system, nth, r.lo != nullptr, &r, ncta, s, nullptr);
 }

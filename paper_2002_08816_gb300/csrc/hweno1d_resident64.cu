@@ -409,10 +409,9 @@ size_t resident64_halo_words(int system, int ncta) {
   return (size_t)ncta * 2 * 6 * (system == 0 ? 1 : 3) * 4;
 }
 
-cudaError_t launch_resident64(const Resident1DArgs& r, int ncta, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(r.halo, 0, sizeof(u64) * resident64_halo_words(r.a.system, ncta), s);
-  if (e == cudaSuccess)
-    e = cudaMemsetAsync(r.entries, 0, sizeof(u64) * resident64_entry_words(ncta), s);
+cudaError_t launch_resident64(const Resident1DArgs& r, int ncta, double t_final, cudaStream_t s) {
+  const cudaError_t e = launch_start_run(r.a.sc, t_final, r.halo, resident64_halo_words(r.a.system, ncta),
+                                         r.entries, resident64_entry_words(ncta), s);
   if (e != cudaSuccess) return e;
   if (r.tile <= kSmallT)
     return r.a.system == 0 ? launch_t<1, kSmallT, kSmallN>(r, ncta, s)

@@ -335,7 +335,7 @@ cudaError_t prepare_resident(hweno_ctx* h, int nth) {
 
 // nsteps Runge-Kutta steps of a 1D handle in one resident launch (silent_cta,
 // polls: the failure-detection self-test; -1 and 2^21 otherwise).
-cudaError_t enqueue_resident1d(hweno_ctx* h, int nsteps, cudaStream_t s, int silent_cta = -1,
+cudaError_t enqueue_resident1d(hweno_ctx* h, int nsteps, double t_final, cudaStream_t s, int silent_cta = -1,
                                unsigned polls = 1u << 21) {
   hw::Resident1DArgs r;
   memset(&r, 0, sizeof(r));
@@ -353,7 +353,7 @@ cudaError_t enqueue_resident1d(hweno_ctx* h, int nsteps, cudaStream_t s, int sil
   r.polls = polls;
   r.silent_cta = silent_cta;
   r.lo = h->comp ? h->Ulo : nullptr;
-  return hw::launch_resident1d(r, h->res_nth, h->res_ncta, s);
+  return hw::launch_resident1d(r, h->res_nth, h->res_ncta, t_final, s);
 }
 
 // nsteps steps as launches of at most 2^29 (a resident run counts its stages in 32
@@ -388,7 +388,7 @@ cudaError_t enqueue_cluster1d(hweno_ctx* h, int nsteps, cudaStream_t s) {
 }
 
 // nsteps Runge-Kutta steps of an FP64 handle in one resident launch.
-cudaError_t enqueue_resident64(hweno_ctx* h, int nsteps, cudaStream_t s) {
+cudaError_t enqueue_resident64(hweno_ctx* h, int nsteps, double t_final, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   if (!h->halo64)
     e = cudaMalloc(&h->halo64, sizeof(unsigned long long) * hw::resident64_halo_words(h->cfg.system, h->ncta64));
@@ -410,7 +410,7 @@ cudaError_t enqueue_resident64(hweno_ctx* h, int nsteps, cudaStream_t s) {
   r.alpha_word = h->entries64 + hw::resident64_entry_words(h->ncta64) - 4;
   r.polls = 1u << 21;
   r.silent_cta = -1;
-  return hw::launch_resident64(r, h->ncta64, s);
+  return hw::launch_resident64(r, h->ncta64, t_final, s);
 }
 
 cudaError_t enqueue_step(hweno_ctx* h, cudaStream_t s) {
@@ -787,14 +787,12 @@ hweno_status hweno_step(hweno_handle h, int nsteps, double t_final, double* t_ou
   if (!h) return fail(nullptr, HWENO_ERR_ARG, "handle is NULL");
   if (!h->has_state) return fail(h, HWENO_ERR_STATE, "hweno_step before hweno_set_state");
   if (nsteps < 0) return fail(h, HWENO_ERR_ARG, "nsteps must be >= 0");
-  HW_CUDA(h, hw::launch_set_scalars(h->sc, 0, t_final, h->stream));
-  if (h->n_batch > 0)
-    HW_CUDA(h, hw::launch_batch_scalars(h->d_bsc, h->n_batch, 0, t_final, h->stream));
   int left = nsteps;
   if (h->tile_cl > 0 && h->n_batch == 0 && left > 0) {
     // FP32 grids that fit one cluster run there, whatever launch the handle is
     // set to: a stage is then bound by its own latency and not by a launch or a
     // round trip to L2 (Lax on 200 cells: 3.7 us per stage by launches, 2.35 on chip)
+    HW_CUDA(h, hw::launch_set_scalars(h->sc, 0, t_final, h->stream));
     HW_CUDA(h, in_launches(left, [&](int k) { return enqueue_cluster1d(h, k, h->stream); }));
     left = 0;
   }
@@ -802,7 +800,7 @@ hweno_status hweno_step(hweno_handle h, int nsteps, double t_final, double* t_ou
     // FP64 single instances whose tiles fit on the GPU at once run on chip,
     // whatever launch the handle is set to: at every size the FP64 pipe and not
     // the launches bounds them, and the resident run spreads it best
-    cudaError_t e = in_launches(left, [&](int k) { return enqueue_resident64(h, k, h->stream); });
+    cudaError_t e = in_launches(left, [&](int k) { return enqueue_resident64(h, k, t_final, h->stream); });
     if (e == cudaSuccess) {
       left = 0;
     } else if (e == cudaErrorCooperativeLaunchTooLarge) {
@@ -819,7 +817,7 @@ hweno_status hweno_step(hweno_handle h, int nsteps, double t_final, double* t_ou
     const int nth = h->persist1d == 2 ? h->nth1d : 256;
     if (h->res_nth != nth) HW_CUDA(h, prepare_resident(h, nth));
     if (h->res_tile > 0) {
-      cudaError_t e = in_launches(left, [&](int k) { return enqueue_resident1d(h, k, h->stream); });
+      cudaError_t e = in_launches(left, [&](int k) { return enqueue_resident1d(h, k, t_final, h->stream); });
       if (e == cudaErrorCooperativeLaunchTooLarge && h->persist1d != 2) {
         cudaGetLastError();
         h->res_tile = 0;
@@ -828,6 +826,11 @@ hweno_status hweno_step(hweno_handle h, int nsteps, double t_final, double* t_ou
         left = 0;
       }
     }
+  }
+  if (left > 0 || nsteps == 0) {  // (the launches above have set t_final)
+    HW_CUDA(h, hw::launch_set_scalars(h->sc, 0, t_final, h->stream));
+    if (h->n_batch > 0)
+      HW_CUDA(h, hw::launch_batch_scalars(h->d_bsc, h->n_batch, 0, t_final, h->stream));
   }
   if (h->dim == 1 && h->persist1d == 1 && h->esize == 8) {  // (FP32: by stages, below)
     if (left > 0) HW_CUDA(h, enqueue_run1d(h, left, h->stream));
@@ -1445,8 +1448,7 @@ hweno_status hweno_check_resident(hweno_handle h, int nsteps, int silent_cta, un
     return fail(h, HWENO_ERR_ARG,
                 "hweno_check_resident: need nsteps >= 1, -1 <= silent_cta < CTAs, polls >= 1");
   if (h->res_nth != h->nth1d) HW_CUDA(h, prepare_resident(h, h->nth1d));
-  HW_CUDA(h, hw::launch_set_scalars(h->sc, 0, -1.0, h->stream));
-  HW_CUDA(h, in_launches(nsteps, [&](int k) { return enqueue_resident1d(h, k, h->stream, silent_cta, polls); }));
+  HW_CUDA(h, in_launches(nsteps, [&](int k) { return enqueue_resident1d(h, k, -1.0, h->stream, silent_cta, polls); }));
   hw::DevScalars host;
   return check_scalars(h, h->sc, &host);  // HWENO_ERR_TIMEOUT when a wait ran out
 }

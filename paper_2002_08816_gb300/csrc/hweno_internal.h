@@ -255,8 +255,8 @@ cudaError_t launch_split_pairs(const void* src, void* hi, float* lo, int C, int 
                                cudaStream_t s);
 cudaError_t launch_join_pairs(const void* hi, const float* lo, double* out, int C, int M, int n,
                               cudaStream_t s);
-// Zeroes the exchange words, then launches.
-cudaError_t launch_resident1d(const Resident1DArgs& r, int nth, int ncta, cudaStream_t s);
+// Sets t_final in the scalars and zeroes the exchange words, then launches.
+cudaError_t launch_resident1d(const Resident1DArgs& r, int nth, int ncta, double t_final, cudaStream_t s);
 
 // The resident run of a small grid (FP32, HWENO_FP32C): its CTAs are one
 // thread-block cluster, or a single CTA, and exchange through shared memory; its
@@ -271,7 +271,7 @@ cudaError_t launch_cluster1d(const Resident1DArgs& r, int ncta, cudaStream_t s);
 cudaError_t resident64_geometry(int n, int* tile, int* ncta);
 size_t resident64_entry_words(int ncta);
 size_t resident64_halo_words(int system, int ncta);
-cudaError_t launch_resident64(const Resident1DArgs& r, int ncta, cudaStream_t s);
+cudaError_t launch_resident64(const Resident1DArgs& r, int ncta, double t_final, cudaStream_t s);
 
 // Cooperative launch of min(ntile, co-resident CTAs) CTAs.
 cudaError_t launch_run1d(const Run1DArgs& r, cudaStream_t s);
@@ -290,6 +290,9 @@ cudaError_t launch_alpha1d(const void* w, void* a_out, int n, int ntile, int sys
 cudaError_t launch_convert(const void* src, int src_fp64, void* dst, int dst_fp64, size_t count,
                            cudaStream_t s);
 cudaError_t launch_set_scalars(DevScalars* sc, int reset, double t_final, cudaStream_t s);
+// The same without a reset, and na words at a and nb at b zeroed (both even).
+cudaError_t launch_start_run(DevScalars* sc, double t_final, unsigned long long* a, size_t na,
+                             unsigned long long* b, size_t nb, cudaStream_t s);
 // out[c] = sum over n cells of base[c * comp_stride + i] in FP64, c < C <= 8, with
 // nblocks partials per component in partials; a fixed summation order.
 cudaError_t launch_totals(const void* base, int fp64, long long comp_stride, int C, long long n,
