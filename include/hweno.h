@@ -261,7 +261,8 @@ hweno_status hweno_check_barrier(int ctas, int meetings, int missing, unsigned p
 
 /* Failure-detection self-test of the resident launch (no counterpart in the
  * paper).  On a handle set to the resident launch (hweno_set_execution(h, 256
- * or 512, 2)) with a state, runs nsteps Runge-Kutta steps in one resident
+ * or 512, 2)), or an FP64 single instance whose steps run resident (6 to about
+ * 76000 cells), with a state, runs nsteps Runge-Kutta steps in one resident
  * launch in which CTA silent_cta (0 <= silent_cta < the launch's CTAs; -1:
  * none) never publishes the maximum wave speed of its outputs, and every wait
  * of the launch gives up after `polls` polls.  With a silent CTA no CTA can
@@ -269,7 +270,7 @@ hweno_status hweno_check_barrier(int ctas, int meetings, int missing, unsigned p
  * word and leaves, the state is not written, and the result is
  * HWENO_ERR_TIMEOUT; the context stays usable (hweno_set_state resets the
  * status).  With silent_cta = -1 it is an ordinary run (HWENO_OK).  Waits for
- * the stream.  HWENO_ERR_ARG for another launch kind or invalid arguments,
+ * the stream.  HWENO_ERR_ARG for another launch or invalid arguments,
  * HWENO_ERR_STATE before hweno_set_state. */
 hweno_status hweno_check_resident(hweno_handle h, int nsteps, int silent_cta, unsigned polls);
 

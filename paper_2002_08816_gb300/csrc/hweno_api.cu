@@ -387,8 +387,10 @@ cudaError_t enqueue_cluster1d(hweno_ctx* h, int nsteps, cudaStream_t s) {
   return hw::launch_cluster1d(r, h->ncta_cl, s);
 }
 
-// nsteps Runge-Kutta steps of an FP64 handle in one resident launch.
-cudaError_t enqueue_resident64(hweno_ctx* h, int nsteps, double t_final, cudaStream_t s) {
+// nsteps Runge-Kutta steps of an FP64 handle in one resident launch (silent_cta,
+// polls: the failure-detection self-test).
+cudaError_t enqueue_resident64(hweno_ctx* h, int nsteps, double t_final, cudaStream_t s, int silent_cta = -1,
+                               unsigned polls = 1u << 21) {
   cudaError_t e = cudaSuccess;
   if (!h->halo64)
     e = cudaMalloc(&h->halo64, sizeof(unsigned long long) * hw::resident64_halo_words(h->cfg.system, h->ncta64));
@@ -408,8 +410,8 @@ cudaError_t enqueue_resident64(hweno_ctx* h, int nsteps, double t_final, cudaStr
   r.halo = h->halo64;
   r.entries = h->entries64;
   r.alpha_word = h->entries64 + hw::resident64_entry_words(h->ncta64) - 4;
-  r.polls = 1u << 21;
-  r.silent_cta = -1;
+  r.polls = polls;
+  r.silent_cta = silent_cta;
   return hw::launch_resident64(r, h->ncta64, t_final, s);
 }
 
@@ -1441,14 +1443,17 @@ hweno_status hweno_check_barrier(int ctas, int meetings, int missing, unsigned p
 
 hweno_status hweno_check_resident(hweno_handle h, int nsteps, int silent_cta, unsigned polls) {
   if (!h) return fail(nullptr, HWENO_ERR_ARG, "handle is NULL");
-  if (h->dim != 1 || h->persist1d != 2 || h->res_tile == 0)
+  const bool fp64 = h->n_batch == 0 && h->tile64 > 0;  // resident under every choice
+  if (!fp64 && (h->dim != 1 || h->persist1d != 2 || h->res_tile == 0))
     return fail(h, HWENO_ERR_ARG, "hweno_check_resident: set the resident launch first");
   if (!h->has_state) return fail(h, HWENO_ERR_STATE, "hweno_check_resident before hweno_set_state");
-  if (nsteps < 1 || silent_cta < -1 || silent_cta >= h->res_ncta || polls < 1u)
+  if (nsteps < 1 || silent_cta < -1 || silent_cta >= (fp64 ? h->ncta64 : h->res_ncta) || polls < 1u)
     return fail(h, HWENO_ERR_ARG,
                 "hweno_check_resident: need nsteps >= 1, -1 <= silent_cta < CTAs, polls >= 1");
-  if (h->res_nth != h->nth1d) HW_CUDA(h, prepare_resident(h, h->nth1d));
-  HW_CUDA(h, in_launches(nsteps, [&](int k) { return enqueue_resident1d(h, k, -1.0, h->stream, silent_cta, polls); }));
+  HW_CUDA(h, in_launches(nsteps, [&](int k) {
+            return fp64 ? enqueue_resident64(h, k, -1.0, h->stream, silent_cta, polls)
+                        : enqueue_resident1d(h, k, -1.0, h->stream, silent_cta, polls);
+          }));
   hw::DevScalars host;
   return check_scalars(h, h->sc, &host);  // HWENO_ERR_TIMEOUT when a wait ran out
 }

@@ -51,3 +51,43 @@ def _check(prec, nx, threads, limits, silent):
 @pytest.mark.parametrize("silent", [-1, 3])
 def test_fp32_waits_of_a_few_polls_end(prec, nx, threads, silent):
     _check(prec, nx, threads, (1, 2, 3, 5, 9, 17, 40, 100, 300, 1000), silent)
+
+
+@pytest.mark.parametrize("nx", [200, 8001, 65536])  # 26-cell tiles, and more cells to a tile
+@pytest.mark.parametrize("silent", [-1, 3])
+def test_fp64_waits_of_a_few_polls_end(nx, silent):
+    _check(H.HWENO_FP64, nx, 0, (1, 2, 3, 5, 9, 17, 40, 100, 300, 1000), silent)
+
+
+@pytest.mark.parametrize("nx,silent", [(200, 0), (8001, 17), (65536, 151)])
+def test_fp64_run_gives_up_when_a_cta_never_publishes(nx, silent):
+    """Every wait for alpha runs out: a status, nothing written, and the handle
+    then steps as a batch of one does (by stage launches)."""
+    import torch
+    u = mixed_euler(nx, 4)
+    cfg = H.make_config(1, H.HWENO_EULER, nx, bc=H.HWENO_BC_OUTFLOW, cfl=0.5, precision=H.HWENO_FP64)
+    stream = torch.cuda.current_stream().cuda_stream
+    got, back = np.empty_like(u), np.empty_like(u)
+    h = H.hweno_create(cfg, stream)
+    try:
+        H.hweno_set_state(h, u.ctypes.data, H.HWENO_FP64, False)
+        assert H.hweno_check_resident(h, 3, silent, 1 << 14) == H.HWENO_ERR_TIMEOUT
+        H.hweno_get_state(h, back.ctypes.data, H.HWENO_FP64, False)
+        assert np.array_equal(back, u)
+        with pytest.raises(H.HwenoError):
+            H.hweno_check_resident(h, 3, 1000, 1 << 14)
+        H.hweno_set_state(h, u.ctypes.data, H.HWENO_FP64, False)
+        assert H.hweno_check_resident(h, 4, -1, 1 << 21) == H.HWENO_OK
+        H.hweno_get_state(h, got.ctypes.data, H.HWENO_FP64, False)
+    finally:
+        H.hweno_destroy(h)
+    h = H.hweno_create_batch(cfg, [nx], stream)
+    try:
+        H.hweno_set_state(h, u.ctypes.data, H.HWENO_FP64, False)
+        H.hweno_step(h, 4)
+        H.hweno_get_state(h, back.ctypes.data, H.HWENO_FP64, False)
+        with pytest.raises(H.HwenoError):  # no resident run
+            H.hweno_check_resident(h, 3, -1, 1 << 14)
+    finally:
+        H.hweno_destroy(h)
+    assert np.abs(got - back).sum() <= 1e-12 * np.abs(back).sum()
