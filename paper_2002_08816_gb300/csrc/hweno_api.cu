@@ -33,7 +33,7 @@ struct hweno_ctx {
   // or one resident launch that keeps the tiles on chip (2, FP32 single
   // instance); hweno_autotune chooses
   int nth1d = 256, persist1d = 0;
-  // the resident launch's geometry and cross-CTA buffers (allocated on first use)
+  // the resident launch's geometry and cross-CTA buffers
   int res_nth = 0, res_tile = 0, res_ncta = 0, res_cap = 0;
   unsigned long long* res_halo = nullptr;     // tagged exchange words of the halos
   unsigned long long* res_entries = nullptr;  // and of the per-CTA maxima
@@ -41,7 +41,7 @@ struct hweno_ctx {
   // available)
   int tile_cl = 0, ncta_cl = 0;
   // FP64 single instances: the resident run's geometry (tile64 = 0: not
-  // available) and its cross-CTA buffers (allocated on first use)
+  // available) and its cross-CTA buffers
   int tile64 = 0, ncta64 = 0;
   unsigned long long* halo64 = nullptr;
   unsigned long long* entries64 = nullptr;
@@ -391,12 +391,6 @@ cudaError_t enqueue_cluster1d(hweno_ctx* h, int nsteps, cudaStream_t s) {
 // polls: the failure-detection self-test).
 cudaError_t enqueue_resident64(hweno_ctx* h, int nsteps, double t_final, cudaStream_t s, int silent_cta = -1,
                                unsigned polls = 1u << 21) {
-  cudaError_t e = cudaSuccess;
-  if (!h->halo64)
-    e = cudaMalloc(&h->halo64, sizeof(unsigned long long) * hw::resident64_halo_words(h->cfg.system, h->ncta64));
-  if (e == cudaSuccess && !h->entries64)
-    e = cudaMalloc(&h->entries64, sizeof(unsigned long long) * hw::resident64_entry_words(h->ncta64));
-  if (e != cudaSuccess) return e;
   hw::Resident1DArgs r;
   memset(&r, 0, sizeof(r));
   r.a = base_args(h);
@@ -715,9 +709,18 @@ hweno_status hweno_create(const hweno_config* cfg, void* cuda_stream, hweno_hand
     hweno_destroy(h);
     return fail(nullptr, HWENO_ERR_CUDA, msg);
   }
-  if (h->dim == 1)
-    e = h->esize == 8 ? hw::resident64_geometry(h->n, &h->tile64, &h->ncta64)
-                      : hw::cluster1d_geometry(cfg->system, h->comp, h->n, &h->tile_cl, &h->ncta_cl);
+  // the resident launches' geometries, and their buffers now, so that a step
+  // allocates nothing (the first one may be captured into a caller's graph)
+  if (h->dim == 1 && h->esize == 8) {
+    e = hw::resident64_geometry(h->n, &h->tile64, &h->ncta64);
+    if (e == cudaSuccess && h->tile64 > 0)
+      e = cudaMalloc(&h->halo64, sizeof(unsigned long long) * hw::resident64_halo_words(cfg->system, h->ncta64));
+    if (e == cudaSuccess && h->tile64 > 0)
+      e = cudaMalloc(&h->entries64, sizeof(unsigned long long) * hw::resident64_entry_words(h->ncta64));
+  } else if (h->dim == 1) {
+    e = hw::cluster1d_geometry(cfg->system, h->comp, h->n, &h->tile_cl, &h->ncta_cl);
+    if (e == cudaSuccess && h->tile_cl == 0) e = prepare_resident(h, 256);
+  }
   if (e != cudaSuccess) {
     std::string msg = std::string("resident launch: ") + cudaGetErrorString(e);
     hweno_destroy(h);
@@ -838,6 +841,12 @@ hweno_status hweno_step(hweno_handle h, int nsteps, double t_final, double* t_ou
     if (left > 0) HW_CUDA(h, enqueue_run1d(h, left, h->stream));
     left = 0;
   }
+  // a caller that captures the stream gets the stages themselves (an instantiated
+  // graph cannot be launched into a capture)
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (left > 0) HW_CUDA(h, cudaStreamIsCapturing(h->stream, &capturing));
+  if (capturing == cudaStreamCaptureStatusActive)
+    for (; left > 0; --left) HW_CUDA(h, enqueue_step(h, h->stream));
   if (left >= kGraphSteps) {
     if (!h->g_many) {
       hweno_status st = build_graph(h, kGraphSteps, &h->g_many);
