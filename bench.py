@@ -309,7 +309,9 @@ def run_1d(H, s, stream, u0, prec, steps, warmup, flush, sampler=None, autotune=
     # this workload (untimed)
     H.hweno_set_state(h, dev_in.data_ptr(), sdt, True)
     choice = H.hweno_autotune(h, 100) if autotune else (256, 0)
-    choice = (choice[0], 2)  # this grid runs resident under every choice, FP64 too
+    # this grid runs resident under every choice; in FP64, where that is all it can
+    # do, the tuner leaves the handle's 256 threads, which are also the run's
+    choice = (choice[0], 2)
     for _ in range(warmup):
         one_step()
     torch.cuda.synchronize()

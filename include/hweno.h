@@ -231,17 +231,21 @@ hweno_status hweno_rhs_vjp(hweno_handle h, const void* in, const uint8_t* flags,
                            double alpha_y, const void* lam, void* grad);
 
 /* Chooses how a 1D handle (single instance or batch) runs its steps among the
- * choices of hweno_set_execution.  Each candidate advances the current state
- * nsteps_trial steps once untimed (which builds its graphs) and then twice
- * timed with CUDA events on the handle's stream; the one with the fastest trial
- * is kept for later calls; the state, time, counters and wave-speed slots are
- * restored afterwards.  The paper has no counterpart (it fixes no hardware
- * mapping).  choice_out (nullable, 2 ints) receives the threads per CTA and the
- * launch kind (0 graphs, 1 persistent, 2 resident).  New handles start with 256
- * threads and kind 0 (HWENO_FP32C: kind 2, the only one it has).  A single FP32
- * or HWENO_FP32C instance that runs resident under every choice is timed with 256
- * and 512 threads of kind 2.  Waits for the stream; HWENO_ERR_ARG for 2D
- * handles, HWENO_ERR_STATE before set_state. */
+ * choices of hweno_set_execution whose launches differ.  Each advances the
+ * current state nsteps_trial steps once untimed (which builds its graphs) and
+ * then twice timed with CUDA events on the handle's stream; the one with the
+ * fastest trial is kept for later calls; the state, time, counters and
+ * wave-speed slots are restored afterwards.  The paper has no counterpart (it
+ * fixes no hardware mapping).  choice_out (nullable, 2 ints) receives the
+ * threads per CTA and the launch kind (0 graphs, 1 persistent, 2 resident).
+ * New handles start with 256 threads and kind 0 (HWENO_FP32C: kind 2, the only
+ * one it has).  Nothing is timed where there is nothing to choose: a single
+ * instance that runs as one cluster, or resident in FP64, under every choice
+ * keeps the choice it has, and a single FP32 instance too large to be resident
+ * gets the stage launches' threads of its size and kind 0.  An FP32 or
+ * HWENO_FP32C instance that runs resident is timed with 256 and 512 threads of
+ * kind 2, FP32 batches with kind 0 only.  Waits for the stream; HWENO_ERR_ARG
+ * for 2D handles, HWENO_ERR_STATE before set_state. */
 hweno_status hweno_autotune(hweno_handle h, int nsteps_trial, int* choice_out);
 
 /* Failure-detection self-test of the grid barrier the persistent launch uses

@@ -16,6 +16,7 @@
 #include <string.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "hweno.h"
@@ -1308,6 +1309,33 @@ hweno_status hweno_autotune(hweno_handle h, int nsteps_trial, int* choice_out) {
   if (h->dim != 1) return fail(h, HWENO_ERR_ARG, "hweno_autotune tunes 1D handles");
   if (!h->has_state) return fail(h, HWENO_ERR_STATE, "hweno_autotune before hweno_set_state");
   if (nsteps_trial < 1) return fail(h, HWENO_ERR_ARG, "nsteps_trial must be >= 1");
+  // the choices whose launches differ: none where the instance runs on chip under
+  // every choice (one cluster, or FP64), the resident launch's two thread counts
+  // where only that is open, one stage launch where its threads follow from the
+  // size (a large FP32 instance), and no persistent launch in FP32
+  std::vector<std::pair<int, int>> cand;  // threads, launch kind
+  const bool single = h->n_batch == 0;
+  if (single && (h->tile_cl > 0 || h->tile64 > 0)) {
+  } else if (single && h->esize == 4) {
+    HW_CUDA(h, prepare_resident(h, 256));
+    if (h->res_tile > 0) cand = {{256, 2}, {512, 2}};
+    else cand = {{stage_threads(h), 0}};
+  } else {
+    for (int persist = 0; persist < (h->esize == 4 ? 1 : 2); ++persist)
+      for (int nth : {128, 256, 512}) cand.push_back({nth, persist});
+  }
+  if (cand.size() < 2) {
+    if (!cand.empty()) {
+      const hweno_status st = hweno_set_execution(h, cand[0].first, cand[0].second);
+      if (st != HWENO_OK) return st;
+    }
+    if (choice_out) {
+      choice_out[0] = h->nth1d;
+      choice_out[1] = h->persist1d;
+    }
+    hw::DevScalars sc;
+    return check_scalars(h, h->sc, &sc);
+  }
   const size_t sbytes = h->elems * h->esize;
   const size_t nslot = h->n_batch > 2 * hw::kAlphaSlots ? (size_t)h->n_batch : 2 * hw::kAlphaSlots;
   const size_t pbytes = sizeof(double) * nslot;
@@ -1352,54 +1380,44 @@ hweno_status hweno_autotune(hweno_handle h, int nsteps_trial, int* choice_out) {
     return cudaSuccess;
   };
   cudaError_t e = copy_all(true);
-  const int cand_nth[3] = {128, 256, 512};
   float best = -1.0f;
   int best_nth = h->nth1d, best_persist = h->persist1d;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
-  // an FP32 instance that runs resident under every choice has only that launch's
-  // threads to choose (the others would time the same run)
-  bool res_only = h->comp;
-  if (e == cudaSuccess && !res_only && h->n_batch == 0 && h->esize == 4) {
-    e = prepare_resident(h, 256);
-    res_only = e == cudaSuccess && h->res_tile > 0;
-  }
-  for (int persist = res_only ? 2 : 0; persist < 3 && e == cudaSuccess; ++persist) {
-    if (persist == 1 && h->esize == 4) continue;  // FP32: the per-stage launches again
-    for (int ci = res_only ? 1 : 0; ci < 3 && e == cudaSuccess; ++ci) {
-      e = configure(cand_nth[ci], persist);
-      if (e != cudaSuccess) break;
-      if (persist == 2 && h->res_tile == 0) continue;  // not available here
-      // one untimed run of the trial length (it builds every graph the trial
-      // launches, so that no graph instantiation is timed), then the best of
-      // two timed trials
-      hweno_status st = HWENO_OK;
-      float ms = -1.0f;
-      for (int rep = 0; rep < 3 && st == HWENO_OK && e == cudaSuccess; ++rep) {
-        e = copy_all(false);
-        if (e == cudaSuccess && rep > 0) e = cudaEventRecord(e0, s);
-        if (e == cudaSuccess) st = hweno_step(h, nsteps_trial, -1.0, nullptr);
-        if (e == cudaSuccess && rep > 0) e = cudaEventRecord(e1, s);
-        if (e == cudaSuccess && st == HWENO_OK && rep > 0) {
-          float t = 0.0f;
-          e = cudaEventSynchronize(e1);
-          if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
-          if (e == cudaSuccess && (ms < 0.0f || t < ms)) ms = t;
-        }
+  for (size_t ci = 0; ci < cand.size() && e == cudaSuccess; ++ci) {
+    const int nth = cand[ci].first, persist = cand[ci].second;
+    e = configure(nth, persist);
+    if (e != cudaSuccess) break;
+    if (persist == 2 && h->res_tile == 0) continue;  // not available here
+    // one untimed run of the trial length (it builds every graph the trial
+    // launches, so that no graph instantiation is timed), then the best of
+    // two timed trials
+    hweno_status st = HWENO_OK;
+    float ms = -1.0f;
+    for (int rep = 0; rep < 3 && st == HWENO_OK && e == cudaSuccess; ++rep) {
+      e = copy_all(false);
+      if (e == cudaSuccess && rep > 0) e = cudaEventRecord(e0, s);
+      if (e == cudaSuccess) st = hweno_step(h, nsteps_trial, -1.0, nullptr);
+      if (e == cudaSuccess && rep > 0) e = cudaEventRecord(e1, s);
+      if (e == cudaSuccess && st == HWENO_OK && rep > 0) {
+        float t = 0.0f;
+        e = cudaEventSynchronize(e1);
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
+        if (e == cudaSuccess && (ms < 0.0f || t < ms)) ms = t;
       }
-      if (e != cudaSuccess) break;
-      if (st != HWENO_OK) {
-        cudaFree(save);
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        return st;
-      }
-      if (best < 0.0f || ms < best) {
-        best = ms;
-        best_nth = cand_nth[ci];
-        best_persist = persist;
-      }
+    }
+    if (e != cudaSuccess) break;
+    if (st != HWENO_OK) {
+      cudaFree(save);
+      cudaEventDestroy(e0);
+      cudaEventDestroy(e1);
+      return st;
+    }
+    if (best < 0.0f || ms < best) {
+      best = ms;
+      best_nth = nth;
+      best_persist = persist;
     }
   }
   if (e == cudaSuccess) e = configure(best_nth, best_persist);
