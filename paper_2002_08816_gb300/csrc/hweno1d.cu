@@ -363,7 +363,9 @@ cudaError_t launch_stage1d_b(const Stage1DArgs& a, cudaStream_t s) {
     if (a.nth == 32) return launch_stage1d_n<R, C, BATCH, 32>(a, s);
   }
   if (a.nth == 128) return launch_stage1d_n<R, C, BATCH, 128>(a, s);
-  if (a.nth == 512) return launch_stage1d_n<R, C, BATCH, 512>(a, s);
+  if constexpr (sizeof(R) == 8 || BATCH) {  // (one FP32 instance: 128 or 256 by its size)
+    if (a.nth == 512) return launch_stage1d_n<R, C, BATCH, 512>(a, s);
+  }
   return launch_stage1d_n<R, C, BATCH, 256>(a, s);
 }
 

@@ -64,7 +64,7 @@ __device__ __forceinline__ T ldx(const T* p) {
 
 template <typename R, int C, int NTH>
 struct Smem1D {
-  static constexpr int T = NTH - 2 * H, NW = NTH / 32;
+  static constexpr int T = NTH - 2 * H;
   R u[C][2][T + 2 * H];  // stage input, cells base-3 .. base+T+2
   R vl[C][T + 4];        // modified first moments, cells base-2 .. base+T+1
   R fm[C][T + 2];        // u^+_{i-1/2}, cells base-1 .. base+T
@@ -72,8 +72,6 @@ struct Smem1D {
   R ffm[C][T + 2];       // f(u^+_{i-1/2})
   R ffp[C][T + 2];       // f(u^-_{i+1/2})
   uint8_t fl[T + 4];     // flags, cells base-2 .. base+T+1
-  R red[NW];
-  int cnt[NW];
   R alpha, dt;           // from the scalar warp, in the kernel's precision
 };
 

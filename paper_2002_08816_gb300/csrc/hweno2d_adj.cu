@@ -779,7 +779,7 @@ __global__ void __launch_bounds__(NT) adj2d_pass_kernel(Adj2DArgs a) {
 // five data Step 1 read) to the adjoints kernel B wrote.
 template <typename R, int C>
 __device__ __noinline__ void fix_tile(const Adj2DArgs& a, int tile) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];  // (one declaration, one alignment)
   SmemB<R, C>& sm = *reinterpret_cast<SmemB<R, C>*>(smem_raw);
   const int tid = threadIdx.x;
   const int nx = a.nx, ny = a.ny;

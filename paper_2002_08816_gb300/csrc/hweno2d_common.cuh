@@ -221,11 +221,6 @@ template <int NG, typename R>
 __device__ __forceinline__ void p0_faces(const R* d, R* o) {
   if constexpr (NG == 3) hw2::p0_faces_ng3(d, o); else hw2::p0_faces_ng2(d, o);
 }
-// The same map on two components of a cell at once (packed FP32).
-template <int NG>
-__device__ __forceinline__ void p0_faces_x2(const float2* d, float2* o) {
-  if constexpr (NG == 3) hw2::p0_faces_ng3_x2(d, o); else hw2::p0_faces_ng2_x2(d, o);
-}
 // The linear p0 of one component (T = float, double) or of two at once (float2)
 // from its parity classes s (hw2::p0_classes of the 19 data): the 2 NG values
 // on the left and right faces, on the bottom and top faces, and the NG^2

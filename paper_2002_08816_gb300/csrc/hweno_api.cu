@@ -603,9 +603,8 @@ hw::Adj2DArgs base_adj_args(const hweno_ctx* h) {
   return a;
 }
 
-// The tiles of every batch instance for stage CTAs of nth threads
-// (stage1d_cells per tile): tile -> instance and first cell, each instance's replaces
-// the previous tiling.
+// The tiles of every batch instance for stage CTAs of nth threads (stage1d_cells
+// per tile), a record each; replaces the previous tiling.
 cudaError_t batch_tiles(hweno_ctx* h, int nth) {
   const int T = hw::stage1d_cells(h->cfg.precision == HWENO_FP64, nth);
   std::vector<hw::BatchTile> tiles;

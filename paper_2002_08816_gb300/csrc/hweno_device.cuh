@@ -72,14 +72,10 @@ struct DevScalars {
 };
 static_assert(sizeof(DevScalars) == 64, "one 64-byte block");
 
-// dt and rem in the kernel's precision
+// dt in the kernel's precision
 template <typename R>
 __device__ __forceinline__ R& sc_dt(DevScalars* s) {
   if constexpr (sizeof(R) == 4) return s->dt_f; else return s->dt;
-}
-template <typename R>
-__device__ __forceinline__ R sc_rem(const DevScalars* s) {
-  if constexpr (sizeof(R) == 4) return s->rem_f; else return s->rem;
 }
 
 // Maximum of a non-negative value into a slot: for x >= 0 the order of the
@@ -203,23 +199,6 @@ __device__ __forceinline__ int list_append(int* count, unsigned short* list, int
   const int q = base + __popc(vote & ((1u << lane) - 1u));
   if (q < cap) list[q] = (unsigned short)item;
   return q;
-}
-
-template <int NT>
-__device__ __forceinline__ double block_max(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  v = (threadIdx.x < NT / 32) ? red[threadIdx.x] : 0.0;
-  if (w == 0)
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if (threadIdx.x == 0) red[0] = v;
-  __syncthreads();
-  v = red[0];
-  __syncthreads();
-  return v;
 }
 
 // Finiteness; FP64 by the exponent's bits (no FP64 instruction).
