@@ -15,7 +15,8 @@ namespace hw {
 
 // x / rho from ir = 1 / rho rounded: FP32 the product (approximate, as ir); FP64
 // with one Newton correction of the quotient by its remainder (Markstein: the
-// correctly rounded quotient), so that several quotients by one rho cost 3 FP64
+// correctly rounded quotient, bit for bit IEEE division's while x, rho, ir and the
+// remainder are normal numbers), so that several quotients by one rho cost 3 FP64
 // instructions each beside 5.4 for ir instead of 8.5 each.
 __device__ __forceinline__ float quotient(float x, float, float ir) { return x * ir; }
 __device__ __forceinline__ double quotient(double x, double rho, double ir) {
