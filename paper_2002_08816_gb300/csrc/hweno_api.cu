@@ -659,7 +659,9 @@ void hweno_default_config(hweno_config* cfg, int dim, int system) {
   cfg->precision = HWENO_FP32;
 }
 
-hweno_status hweno_create(const hweno_config* cfg, void* cuda_stream, hweno_handle* out) {
+// A handle for the cells of cfg; batch: of several instances, whose steps have no
+// resident launch.
+static hweno_status create_handle(const hweno_config* cfg, void* cuda_stream, bool batch, hweno_handle* out) {
   if (!out) return fail(nullptr, HWENO_ERR_ARG, "out is NULL");
   hweno_status st = validate(cfg);
   if (st != HWENO_OK) return st;
@@ -711,13 +713,13 @@ hweno_status hweno_create(const hweno_config* cfg, void* cuda_stream, hweno_hand
   }
   // the resident launches' geometries, and their buffers now, so that a step
   // allocates nothing (the first one may be captured into a caller's graph)
-  if (h->dim == 1 && h->esize == 8) {
+  if (h->dim == 1 && !batch && h->esize == 8) {
     e = hw::resident64_geometry(h->n, &h->tile64, &h->ncta64);
     if (e == cudaSuccess && h->tile64 > 0)
       e = cudaMalloc(&h->halo64, sizeof(unsigned long long) * hw::resident64_halo_words(cfg->system, h->ncta64));
     if (e == cudaSuccess && h->tile64 > 0)
       e = cudaMalloc(&h->entries64, sizeof(unsigned long long) * hw::resident64_entry_words(h->ncta64));
-  } else if (h->dim == 1) {
+  } else if (h->dim == 1 && !batch) {
     e = hw::cluster1d_geometry(cfg->system, h->comp, h->n, &h->tile_cl, &h->ncta_cl);
     if (e == cudaSuccess && h->tile_cl == 0) e = prepare_resident(h, 256);
   }
@@ -739,6 +741,10 @@ hweno_status hweno_create(const hweno_config* cfg, void* cuda_stream, hweno_hand
   }
   *out = h;
   return HWENO_OK;
+}
+
+hweno_status hweno_create(const hweno_config* cfg, void* cuda_stream, hweno_handle* out) {
+  return create_handle(cfg, cuda_stream, false, out);
 }
 
 hweno_status hweno_set_state(hweno_handle h, const void* moments, int dtype, int on_device) {
@@ -1006,7 +1012,7 @@ hweno_status hweno_create_batch(const hweno_config* cfg, int n_batch, const int*
   if (st != HWENO_OK) return st;
   c.nx = (int)total;
   hweno_handle h = nullptr;
-  st = hweno_create(&c, cuda_stream, &h);
+  st = create_handle(&c, cuda_stream, true, &h);
   if (st != HWENO_OK) return st;
   h->cfg.nx = (int)total;
   h->n_batch = n_batch;
