@@ -122,7 +122,8 @@ hweno_status hweno_set_state(hweno_handle h, const void* moments, int dtype, int
  * stream.  dt = cfl * dx / alpha (1D) or cfl / (alpha_x/dx + alpha_y/dy) (2D)
  * from the state at the start of each step, computed and kept on the device;
  * with t_final > 0 the step is clipped so that t does not pass t_final and
- * steps after t_final do nothing.  t_out NULL: returns without waiting.
+ * steps after t_final do nothing.  t_out NULL: returns without waiting (a
+ * caller may then capture the stream into a CUDA graph).
  * t_out non-NULL: waits for the stream, stores the time reached, and returns
  * HWENO_ERR_NONPHYSICAL if any stage saw a non-finite or non-physical value. */
 hweno_status hweno_step(hweno_handle h, int nsteps, double t_final, double* t_out);

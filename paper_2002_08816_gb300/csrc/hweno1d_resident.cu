@@ -31,8 +31,8 @@
 // Every wait is bounded (r.polls polls; the library passes 2^21, about a
 // second): a CTA whose wait runs out sets ST_TIMEOUT and leaves, so the others
 // run out too and the launch ends with a status the host reads.  A self-test
-// (hweno_check_resident) names a CTA that never publishes its maximum.  The arithmetic of a cell is that of the
-// per-stage kernel (hweno1d_stage.cuh): the same helpers in the same order.
+// (hweno_check_resident) names a CTA that never publishes its maximum.  The
+// arithmetic of a cell is that of the helpers in hweno1d_stage.cuh.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

@@ -17,9 +17,10 @@
 //
 // Measured (GB300, one pass of set_state, steps, get_state, before: per-stage or
 // persistent launches with a cell per thread): 400 cells with shocks, 60 steps
-// 9.57 -> 2.86 ms (15.9 us per stage); 65536 cells, 10 steps 2.33 -> 1.20 ms
-// (40 us per stage; the FP64 instructions alone would take ~28).  One CTA of 432
-// cells per SM instead of two of 216: 12 % slower.
+// 9.59 -> 2.87 ms (15.9 us per stage); 65536 cells, 10 steps 2.33 -> 1.19 ms
+// (36.8 us per stage alone, the FP64 pipe active 64 % of it; over 2000 steps, with
+// shocks formed, 69 -> 67 us per stage).  One CTA of 432 cells per SM instead of two
+// of 216: 12 % slower.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
