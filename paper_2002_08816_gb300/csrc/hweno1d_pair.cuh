@@ -12,10 +12,11 @@
 // keeps its slot's data from the flags to the combination in registers (the
 // interior values and their fluxes never leave them).
 //
-// Troubled cells and the cells next to them are listed, and their
+// Euler: troubled cells and the cells next to them are listed, and their
 // characteristic work runs as one field per lane, ten cells to a warp: with
 // thread-own work a warp with one troubled cell ran all three fields' chains
-// for its other 31 lanes' sake.
+// for its other 31 lanes' sake.  Burgers has one field: the thread that holds the
+// cell does it (two barriers and a list less).
 //
 // Measured (GB300, us per stage, a cell per thread -> this): 512 instances of
 // 256-16384 cells, 128 threads 62.7 -> 43.3; 1000000 cells 36.5 -> 22.4; 300000
@@ -145,7 +146,7 @@ __device__ __forceinline__ bool troubled_half(const float2* um, const float2* u0
 
 // The limiter of the listed troubled cells: (cell, field) on consecutive lanes.
 template <int C, int NTH>
-__device__ __noinline__ void limit_listed(SmemPair<C, NTH>& sm, int tid, float gas, float g0, float g1,
+__device__ __forceinline__ void limit_listed(SmemPair<C, NTH>& sm, int tid, float gas, float g0, float g1,
                                           float g2, float eps) {
   constexpr int PW = 32 / C;  // cells a warp takes at once
   const float gam[3] = {g0, g1, g2};
@@ -174,7 +175,7 @@ __device__ __noinline__ void limit_listed(SmemPair<C, NTH>& sm, int tid, float g
 
 // Step 2.1 of the listed cells into P, the same way.
 template <int C, int NTH>
-__device__ __noinline__ void hweno_listed(SmemPair<C, NTH>& sm, int tid, float gas, float g0, float g1,
+__device__ __forceinline__ void hweno_listed(SmemPair<C, NTH>& sm, int tid, float gas, float g0, float g1,
                                           float g2, float eps, int variant) {
   constexpr int PW = 32 / C;
   const float gam[3] = {g0, g1, g2};
@@ -210,6 +211,21 @@ __device__ __noinline__ void hweno_listed(SmemPair<C, NTH>& sm, int tid, float g
       }
     }
   }
+}
+
+// The same two out of line, for the 128-thread build, whose five CTAs per SM cover a
+// call's latency; the others are 3-4 % faster with the work inline (100 instances of
+// 40-400 cells, 256 threads: 4.13 -> 3.99 us per stage; 512 of 256-16384, 128 threads:
+// 42.3 inline 42.5).
+template <int C, int NTH>
+__device__ __noinline__ void limit_call(SmemPair<C, NTH>& sm, int tid, float gas, float g0, float g1, float g2,
+                                        float eps) {
+  limit_listed<C, NTH>(sm, tid, gas, g0, g1, g2, eps);
+}
+template <int C, int NTH>
+__device__ __noinline__ void hweno_call(SmemPair<C, NTH>& sm, int tid, float gas, float g0, float g1, float g2,
+                                        float eps, int variant) {
+  hweno_listed<C, NTH>(sm, tid, gas, g0, g1, g2, eps, variant);
 }
 
 // A tile of 2 (NTH - 6) cells by a CTA of NTH cell threads and the scalar warp
@@ -313,9 +329,13 @@ __device__ __forceinline__ void stage_tile(Stage1DArgs a, const int tile, SmemPa
              (troubled_half<C>(um, u0, up, vm, v0, vp, 1, a.hthr, a.hthr_lo) << 1);
     }
     sm.fl[e] = (uint8_t)flag;
+    if constexpr (C == 1) {  // one field: the thread that holds the cell limits it
+      if (flag & 1) v0[0].x = fld::limit_moment(um[0].x, u0[0].x, up[0].x, vm[0].x, vp[0].x, gam, eps);
+      if (flag & 2) v0[0].y = fld::limit_moment(um[0].y, u0[0].y, up[0].y, vm[0].y, vp[0].y, gam, eps);
+    }
 #pragma unroll
     for (int c = 0; c < C; ++c) sm.vl[c][e] = v0[c];  // (listed cells: replaced below)
-    if (flag) {
+    if (C == 3 && flag) {
       int k = atomicAdd(&sm.ntb, __popc(flag));
       if (flag & 1) sm.tb[k++] = (unsigned short)(2 * e);
       if (flag & 2) sm.tb[k] = (unsigned short)(2 * e + 1);
@@ -323,9 +343,12 @@ __device__ __forceinline__ void stage_tile(Stage1DArgs a, const int tile, SmemPa
   }
   bar_sync(kBarCells, NTH);
   int hwm = 0;  // halves of this thread's slot whose stencil holds a troubled cell
-  const bool any = sm.ntb > 0;  // uniform over the CTA
-  if (any) {
-    limit_listed<C, NTH>(sm, tid, gas, gam[0], gam[1], gam[2], eps);
+  const bool any = C == 1 || sm.ntb > 0;  // uniform over the CTA
+  if constexpr (C == 1) {
+    if (tid < W + 2) hwm = sm.fl[e - 1] | sm.fl[e] | sm.fl[e + 1];
+  } else if (any) {
+    if constexpr (NTH == 128) limit_call<C, NTH>(sm, tid, gas, gam[0], gam[1], gam[2], eps);
+    else limit_listed<C, NTH>(sm, tid, gas, gam[0], gam[1], gam[2], eps);
     if (tid < W + 2) {
       hwm = sm.fl[e - 1] | sm.fl[e] | sm.fl[e + 1];
       if (hwm) {
@@ -335,7 +358,8 @@ __device__ __forceinline__ void stage_tile(Stage1DArgs a, const int tile, SmemPa
       }
     }
     bar_sync(kBarCells, NTH);
-    hweno_listed<C, NTH>(sm, tid, gas, gam[0], gam[1], gam[2], eps, a.variant);
+    if constexpr (NTH == 128) hweno_call<C, NTH>(sm, tid, gas, gam[0], gam[1], gam[2], eps, a.variant);
+    else hweno_listed<C, NTH>(sm, tid, gas, gam[0], gam[1], gam[2], eps, a.variant);
     bar_sync(kBarCells, NTH);
   }
 
@@ -345,8 +369,14 @@ __device__ __forceinline__ void stage_tile(Stage1DArgs a, const int tile, SmemPa
     float2 gm[C], gp[C], f2[NF], f3[NF];
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-      if (any) v0[c] = sm.vl[c][e];
-      p0_pair(um[c], u0[c], up[c], sm.vl[c][e - 1], v0[c], sm.vl[c][e + 1], L[c], Rt[c], gm[c], gp[c]);
+      if (C == 3 && any) v0[c] = sm.vl[c][e];
+      const float2 vm = sm.vl[c][e - 1], vp = sm.vl[c][e + 1];
+      p0_pair(um[c], u0[c], up[c], vm, v0[c], vp, L[c], Rt[c], gm[c], gp[c]);
+      if constexpr (C == 1) {
+        if (hwm & 1) fld::hweno(um[c].x, u0[c].x, up[c].x, vm.x, v0[c].x, vp.x, gam, eps, L[c].x, Rt[c].x);
+        if (hwm & 2) fld::hweno(um[c].y, u0[c].y, up[c].y, vm.y, v0[c].y, vp.y, gam, eps, L[c].y, Rt[c].y);
+        continue;
+      }
       if (hwm & 1) {
         L[c].x = sm.P[0][c][e].x;
         Rt[c].x = sm.P[1][c][e].x;
