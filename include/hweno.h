@@ -239,8 +239,8 @@ hweno_status hweno_rhs_vjp(hweno_handle h, const void* in, const uint8_t* flags,
  * wave-speed slots are restored afterwards.  The paper has no counterpart (it
  * fixes no hardware mapping).  choice_out (nullable, 2 ints) receives the
  * threads per CTA and the launch kind (0 graphs, 1 persistent, 2 resident).
- * New handles start with 256 threads and kind 0 (HWENO_FP32C: kind 2, the only
- * one it has).  Nothing is timed where there is nothing to choose: a single
+ * New handles start with 256 threads (small FP32 batches 128) and kind 0
+ * (HWENO_FP32C: kind 2, the only one it has).  Nothing is timed where there is nothing to choose: a single
  * instance that runs as one cluster, or resident in FP64, under every choice
  * keeps the choice it has, and a single FP32 instance too large to be resident
  * gets the stage launches' threads of its size and kind 0.  An FP32 or

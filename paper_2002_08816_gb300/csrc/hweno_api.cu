@@ -1038,6 +1038,15 @@ hweno_status hweno_create_batch(const hweno_config* cfg, int n_batch, const int*
     cells += nx[b];
   }
   cudaError_t e = cudaMalloc(&h->d_bsc, sizeof(hw::BatchScalars) * n_batch);
+  // FP32 batches of at most one 256-thread tile per SM start with 128 threads: a stage
+  // is then one tile's chain, and two smaller tiles share it (us per stage with 128 /
+  // 256: 64 instances of 40-400 cells 3.72 / 3.96, 100 3.75 / 3.99, 16 of 40-200 3.6
+  // both; 250 of 40-800, on 284 tiles, 5.25 / 5.05)
+  if (h->esize == 4) {
+    long long tiles = 0;
+    for (int b = 0; b < n_batch; ++b) tiles += tiles1d(nx[b], c.precision, 256);
+    if (tiles <= 152) h->nth1d = 128;
+  }
   if (e == cudaSuccess) e = batch_tiles(h, h->nth1d);
   // one alpha slot per instance in each of the three rotating buffers
   for (int r = 0; r < 3 && e == cudaSuccess && n_batch > 2 * hw::kAlphaSlots; ++r) {
