@@ -290,7 +290,10 @@ hweno_status hweno_check_resident(hweno_handle h, int nsteps, int silent_cta, un
  * A single instance whose tiles fit on the GPU at once runs resident under every
  * choice, because nothing else is as fast there: grids of 6 to about 4000 cells
  * in FP32 and HWENO_FP32C as one thread-block cluster, up to about 76000 cells
- * in FP32 and FP64 as one cooperative launch.  The choice then selects among
+ * in FP32 and FP64 as one cooperative launch.  A resident run holds the SMs it
+ * takes (FP32: one per 250 cells up to 38000 cells, all beyond) until it ends, so
+ * that other streams' work shares the rest; many instances at once are best
+ * stepped as a batch.  The choice then selects among
  * the launches of batches, larger grids and grids below 6 cells, and with kind 2
  * the resident launch's threads; a single FP32 instance's stage launches take
  * their threads from its size.  1D handles only; waits for the stream.  All

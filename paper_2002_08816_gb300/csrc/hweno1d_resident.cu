@@ -779,6 +779,14 @@ cudaError_t resident1d_geometry(int system, int nth, bool comp, int n, int* tile
   if (slots > 32 * kMaxEnt) slots = 32 * kMaxEnt;  // the scalar warp polls at most this many
   int t = (int)((n + slots - 1) / slots);
   if (t < 6) t = 6;
+  // FP32, 256 threads, a grid of at most one full tile per SM: the fewest CTAs
+  // instead.  The run is as fast (us per stage with all 304 CTAs / the fewest: 5000
+  // cells 2.67 / 2.62, 20000 2.66 / 2.77, 30000 2.83 / 2.74, 38000 3.61 / 2.85) and
+  // leaves the other SMs to other streams, whose resident runs would wait for its end
+  // (us per stage of all: 16 handles of 5000 cells on 16 streams 43.4 / 5.0, 4 of
+  // 20000 10.7 / 4.5; HWENO_FP32C, 20000 cells alone: 3.19 / 3.45)
+  const int full = (n + nth - 7) / (nth - 6);
+  if (nth == 256 && !comp && full <= nsm) t = std::max(t, (n + full - 1) / full);
   for (; t <= nth - 6; ++t) {
     const int c = (n + t - 1) / t;
     if (c <= slots && n - (c - 1) * t >= 6) {

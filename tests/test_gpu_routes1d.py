@@ -134,3 +134,10 @@ def test_batches(system, bc, prec, choice):
 def test_resident_threads(threads):
     _single(E, OUT, 20011, F32, 10, (threads, 2), chunks=2)
     _single(E, OUT, 20011, F32C, 10, (threads, 2), chunks=2)
+
+
+@pytest.mark.parametrize("prec", [F32, F32C])
+@pytest.mark.parametrize("bc", [OUT, REF, PER])
+@pytest.mark.parametrize("nx", [5251, 37999, 38000, 38001])  # full tiles up to one per SM, then shares of all slots
+def test_resident_tilings(nx, bc, prec):
+    _single(E, bc, nx, prec, 6, chunks=2)
